@@ -16,6 +16,7 @@
 //      close eigenvalues (modified Gram-Schmidt);
 //   7. back-transformation by the Householder reflectors, Y = D L^-T Z.
 // Every loop is bounded by the matrix size; nothing waits on another CTA.
+#include <algorithm>
 #include <cfloat>
 
 #include "internal.h"
@@ -71,19 +72,6 @@ __device__ double block_min(double v, double* red) {
 }
 
 __device__ double block_max(double v, double* red) { return -block_min(-v, red); }
-
-// Number of eigenvalues of the tridiagonal (d, e) below x, in FP32 (used to
-// locate shifts; FP64 is ~60x slower per operation on this part).
-__device__ int sturm_count_f(const float* d, const float* e2, int n, float x, float tiny) {
-  int c = 0;
-  float q = 1.0f;
-  for (int i = 0; i < n; ++i) {
-    q = d[i] - x - ((i > 0) ? __fdividef(e2[i - 1], q) : 0.0f);
-    if (fabsf(q) < tiny) q = -tiny;
-    if (q < 0.0f) ++c;
-  }
-  return c;
-}
 
 // Number of eigenvalues of the tridiagonal (d, e) below x.
 __device__ int sturm_count(const double* d, const double* e, int n, double x, double tiny) {
@@ -588,368 +576,26 @@ __global__ void __launch_bounds__(RR_THREADS) rr_kernel(const RRTask* __restrict
   }
 }
 
-
-// Shared-memory variant for pencils whose n x n working matrix and n x m
-// eigenvector block fit in one CTA's shared memory (n = 3m <= ~150 at m = 48).
-// Same algorithm; every O(n^3) phase runs on shared memory with all threads
-// (right-looking triangular solves, in-place Householder reflectors) and the
-// eigenvalues are found by parallel multisection of the Sturm count.
-constexpr int RRS_THREADS = 512;
-
-__global__ void __launch_bounds__(RRS_THREADS) rr_smem_kernel(const RRTask* __restrict__ tasks) {
-  const RRTask T = tasks[blockIdx.x];
-  if (T.state && !T.state[ST_ACTIVE]) return;
-  if (T.state && (T.state[ST_ERROR] & ERR_TIMEOUT)) {
-    // a wait in this iteration's Gram launch ran out: its products are stale
-    if (threadIdx.x == 0) T.state[ST_ACTIVE] = 0;
-    return;
-  }
-  extern __shared__ __align__(16) double smd[];
-  __shared__ double red[32];
-  __shared__ int sflag;
-  __shared__ double sval[4];
-  const int m = T.m;
-  int n = (T.mode == RR_FIXED) ? T.n_fixed
-          : (T.mode == RR_INITIAL) ? m
-          : (T.state[ST_HAS_P] ? 3 * m : 2 * m);
-  const int bm = (T.mode == RR_FIXED) ? n : m;
-  const int n_out = (T.mode == RR_LOBPCG) ? 3 * m : n;
-  const int nmax = n;  // shared layout is sized for the first attempt
-  double* S = smd;                          // n x n working matrix
-  double* Z = S + (size_t)nmax * nmax;      // n x m eigenvectors
-  double* d = Z + (size_t)nmax * m;         // tridiagonal diagonal
-  double* e = d + nmax;                     // off-diagonal
-  double* scal = e + nmax;                  // equilibration
-  double* ptmp = scal + nmax;               // n scratch
-  double* lam = ptmp + nmax;                // m eigenvalues
-  double* lo_s = lam + m;                   // m interval bounds
-  double* hi_s = lo_s + m;
-  int* cnt = reinterpret_cast<int*>(hi_s + m);  // multisection counts (nt)
-  bool dropped = false;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-
-  for (;;) {
-    RRWork W = carve(T.work, n, m);  // global: L (n x n), tri-solve scratch, cluster starts
-    // 1. B: symmetrise, equilibrate, Cholesky in shared memory
-    for (int idx = tid; idx < n * n; idx += nt) {
-      const int r = idx % n, c = idx / n;
-      const int br = r / bm, bc = c / bm;
-      double b;
-      if (br < bc) b = T.B[r + (size_t)c * T.ld];
-      else if (br > bc) b = T.B[c + (size_t)r * T.ld];
-      else b = 0.5 * (T.B[r + (size_t)c * T.ld] + T.B[c + (size_t)r * T.ld]);
-      S[idx] = b;
-    }
-    if (tid == 0) sflag = 0;
-    __syncthreads();
-    for (int i = tid; i < n; i += nt) {
-      const double bii = S[i + (size_t)i * n];
-      if (!(bii > 0.0) || !isfinite(bii)) {
-        sflag = 1;
-        scal[i] = 0.0;
-      } else {
-        scal[i] = 1.0 / sqrt(bii);
-      }
-    }
-    __syncthreads();
-    for (int idx = tid; idx < n * n; idx += nt) S[idx] *= scal[idx % n] * scal[idx / n];
-    __syncthreads();
-    double pmin = DBL_MAX, pmax = 0.0;
-    for (int k = 0; k < n && !sflag; ++k) {
-      if (tid == 0) {
-        const double p = S[k + (size_t)k * n];
-        if (!(p > 0.0) || !isfinite(p)) {
-          sflag = 1;
-        } else {
-          sval[0] = sqrt(p);
-          S[k + (size_t)k * n] = sval[0];
-        }
-      }
-      __syncthreads();
-      if (sflag) break;
-      const double dk = sval[0];
-      pmin = fmin(pmin, dk);
-      pmax = fmax(pmax, dk);
-      const double inv = 1.0 / dk;
-      for (int i = k + 1 + tid; i < n; i += nt) S[i + (size_t)k * n] *= inv;
-      __syncthreads();
-      const int nk = n - k - 1;
-      for (int t = tid; t < nk * nk; t += nt) {
-        const int jj = t / nk, ii = t - jj * nk;
-        if (ii < jj) continue;
-        const int i = k + 1 + ii, j = k + 1 + jj;
-        S[i + (size_t)j * n] -= S[i + (size_t)k * n] * S[j + (size_t)k * n];
-      }
-      __syncthreads();
-    }
-    bool fail = sflag != 0;
-    // the last LOBPCG resort (X alone) takes any positive-definite B: its
-    // Rayleigh-Ritz re-orthonormalises a block that has drifted
-    const bool last_resort = T.mode == RR_LOBPCG && n == m;
-    const double cond_lim = last_resort ? (T.restart_max > 0 ? 1e6 : 1e300) : T.cond_max;
-    if (!fail && (pmax / pmin) * (pmax / pmin) > cond_lim) fail = true;
-    // read before the barrier: thread 0 updates the count after it
-    const bool can_restart =
-        T.mode == RR_LOBPCG && T.restart_max > 0 && T.state && T.state[ST_NRESTART] < T.restart_max;
-    __syncthreads();
-    if (fail) {
-      if (T.mode == RR_LOBPCG && n == 3 * m) {
-        n = 2 * m;
-        dropped = true;
-        __syncthreads();
-        continue;
-      }
-      if (T.mode == RR_LOBPCG && n == 2 * m) {
-        // [X W] is numerically dependent too (W nearly inside span X or
-        // its columns nearly parallel): Rayleigh-Ritz on X alone, a
-        // rotation of the current block; the next iteration brings a new W
-        n = m;
-        dropped = true;
-        __syncthreads();
-        continue;
-      }
-      if (can_restart) {
-        // no usable pencil, not even X alone: keep X (Y = [I; 0]) and let
-        // the restart step perturb it and drop P (Ritz values unchanged)
-        const int nr = 3 * m;
-        for (int idx = tid; idx < nr * m; idx += nt) {
-          const int r = idx % nr, c = idx / nr;
-          const double y = (r == c) ? 1.0 : 0.0;
-          T.Y[r + (size_t)c * T.ldy] = y;
-          if (T.Yf) T.Yf[r + (size_t)c * T.ldy] = (float)y;
-        }
-        if (tid == 0) {
-          T.state[ST_RESTART] = 1;
-          T.state[ST_NRESTART] += 1;
-          T.state[ST_FALLBACK] += 1;
-        }
-        return;
-      }
-      if (tid == 0 && T.state) {
-        T.state[ST_ERROR] |= ERR_CHOL;
-        T.state[ST_ACTIVE] = 0;
-      }
-      if (tid == 0 && !T.state) T.theta[0] = __longlong_as_double(0x7ff8000000000000LL);
-      return;
-    }
-    for (int idx = tid; idx < n * n; idx += nt) {
-      const int r = idx % n, c = idx / n;
-      const double l = (r >= c) ? S[idx] : 0.0;
-      W.L[idx] = l;                    // L, column-major
-      W.H[c + (size_t)r * n] = l;      // L^T, for the final back-substitution
-    }
-    __syncthreads();
-    // 2. C = L^-1 A L^-T: A into shared memory, two right-looking solves
-    for (int idx = tid; idx < n * n; idx += nt) {
-      const int r = idx % n, c = idx / n;
-      const int br = r / bm, bc = c / bm;
-      double a;
-      if (br < bc) a = T.A[r + (size_t)c * T.ld];
-      else if (br > bc) a = T.A[c + (size_t)r * T.ld];
-      else a = 0.5 * (T.A[r + (size_t)c * T.ld] + T.A[c + (size_t)r * T.ld]);
-      S[idx] = a * scal[r] * scal[c];
-    }
-    __syncthreads();
-    for (int pass = 0; pass < 2; ++pass) {
-      for (int k = 0; k < n; ++k) {
-        const double inv = 1.0 / W.L[k + (size_t)k * n];
-        for (int c = tid; c < n; c += nt) S[k + (size_t)c * n] *= inv;
-        __syncthreads();
-        const int nk = n - k - 1;
-        for (int t = tid; t < nk * n; t += nt) {
-          const int c = t / nk, i = k + 1 + (t - c * nk);
-          S[i + (size_t)c * n] -= W.L[i + (size_t)k * n] * S[k + (size_t)c * n];
-        }
-        __syncthreads();
-      }
-      if (pass == 0) {  // S <- S^T
-        for (int idx = tid; idx < n * n; idx += nt) {
-          const int r = idx % n, c = idx / n;
-          if (r < c) {
-            const double t = S[idx];
-            S[idx] = S[c + (size_t)r * n];
-            S[c + (size_t)r * n] = t;
-          }
-        }
-        __syncthreads();
-      }
-    }
-    for (int idx = tid; idx < n * n; idx += nt) {
-      const int r = idx % n, c = idx / n;
-      if (r < c) {
-        const double v = 0.5 * (S[idx] + S[c + (size_t)r * n]);
-        S[idx] = v;
-        S[c + (size_t)r * n] = v;
-      }
-    }
-    __syncthreads();
-    // 3. Householder tridiagonalisation; reflector k kept in S[k+1.., k]
-    for (int k = 0; k + 2 < n; ++k) {
-      double part = 0.0;
-      for (int i = k + 1 + tid; i < n; i += nt) {
-        const double x = S[i + (size_t)k * n];
-        part += x * x;
-      }
-      const double xx = block_sum(part, red);
-      const double x0 = S[k + 1 + (size_t)k * n];
-      const double alpha = (x0 >= 0.0) ? -sqrt(xx) : sqrt(xx);
-      const double vn2 = xx - 2.0 * alpha * x0 + alpha * alpha;
-      if (tid == 0) {
-        d[k] = S[k + (size_t)k * n];
-        e[k] = (vn2 > 0.0) ? alpha : x0;
-      }
-      __syncthreads();
-      double* v = S + (size_t)k * n;  // column k, rows > k
-      if (!(vn2 > 0.0)) {
-        for (int i = k + 1 + tid; i < n; i += nt) v[i] = 0.0;
-        __syncthreads();
-        continue;
-      }
-      const double inv = 1.0 / sqrt(vn2);
-      for (int i = k + 1 + tid; i < n; i += nt) v[i] = (i == k + 1 ? x0 - alpha : v[i]) * inv;
-      __syncthreads();
-      for (int i = k + 1 + warp; i < n; i += nw) {
-        double s2 = 0.0;
-        for (int j = k + 1 + lane; j < n; j += 32) s2 += S[j + (size_t)i * n] * v[j];
-        s2 = warp_sum(s2);
-        if (lane == 0) ptmp[i] = s2;
-      }
-      __syncthreads();
-      double kp = 0.0;
-      for (int i = k + 1 + tid; i < n; i += nt) kp += v[i] * ptmp[i];
-      const double K = block_sum(kp, red);
-      for (int i = k + 1 + tid; i < n; i += nt) ptmp[i] = 2.0 * ptmp[i] - 2.0 * K * v[i];
-      __syncthreads();
-      const int nk = n - k - 1;
-      for (int t = tid; t < nk * nk; t += nt) {
-        const int jj = t / nk, ii = t - jj * nk;
-        const int i = k + 1 + ii, j = k + 1 + jj;
-        S[i + (size_t)j * n] -= v[i] * ptmp[j] + ptmp[i] * v[j];
-      }
-      __syncthreads();
-    }
-    if (tid == 0) {
-      if (n >= 2) {
-        d[n - 2] = S[n - 2 + (size_t)(n - 2) * n];
-        e[n - 2] = S[n - 1 + (size_t)(n - 2) * n];
-      }
-      d[n - 1] = S[n - 1 + (size_t)(n - 1) * n];
-      e[n - 1] = 0.0;
-      if (n >= 2) S[n - 1 + (size_t)(n - 2) * n] = 0.0;  // no reflector for the last columns
-    }
-    __syncthreads();
-    // 4. eigenvalue shifts: FP32 Sturm bisection, one thread per eigenvalue
-    // (final eigenvalues are FP64 Rayleigh quotients after inverse iteration)
-    double glo = DBL_MAX, ghi = -DBL_MAX, gnorm = 0.0;
-    for (int i = tid; i < n; i += nt) {
-      const double r = (i > 0 ? fabs(e[i - 1]) : 0.0) + (i < n - 1 ? fabs(e[i]) : 0.0);
-      glo = fmin(glo, d[i] - r);
-      ghi = fmax(ghi, d[i] + r);
-      gnorm = fmax(gnorm, fabs(d[i]) + r);
-    }
-    glo = block_min(glo, red);
-    ghi = block_max(ghi, red);
-    gnorm = block_max(gnorm, red);
-    const double eps = DBL_EPSILON;
-    float* df = reinterpret_cast<float*>(cnt);    // n <= RRS_THREADS floats
-    float* ef2 = reinterpret_cast<float*>(ptmp);  // n floats in n doubles
-    for (int i = tid; i < n; i += nt) {
-      df[i] = (float)d[i];
-      ef2[i] = (float)(e[i] * e[i]);
-    }
-    __syncthreads();
-    {
-      const float tinyf = 1e-30f;
-      const float padf = 1e-6f * (float)fmax(gnorm, 1e-30);
-      for (int j = tid; j < m; j += nt) {
-        float lo = (float)glo - padf, hi = (float)ghi + padf;
-        for (int it = 0; it < 40; ++it) {
-          const float mid = 0.5f * (lo + hi);
-          if (!(mid > lo && mid < hi)) break;
-          if (sturm_count_f(df, ef2, n, mid, tinyf) > j)
-            hi = mid;
-          else
-            lo = mid;
-        }
-        lam[j] = 0.5 * ((double)lo + (double)hi);
-      }
-    }
-    __syncthreads();
-    // 5. eigenvectors by inverse iteration; shifts closer than the FP32
-    // location accuracy form clusters, orthogonalised within the cluster
-    tri_eigvecs(d, e, n, m, lam, Z, n, W.cstart, lo_s, hi_s, W.tri, 1e-5 * gnorm, gnorm, red, blockIdx.x);
-    // 6. back-transformation, then Y = D L^-T Z (right-looking)
-    for (int k = n - 3; k >= 0; --k) {
-      const double* v = S + (size_t)k * n;
-      for (int c = warp; c < m; c += nw) {
-        const double* zc = Z + (size_t)c * n;
-        double s4 = 0.0;
-        for (int i = k + 1 + lane; i < n; i += 32) s4 += v[i] * zc[i];
-        s4 = warp_sum(s4);
-        if (lane == 0) ptmp[c] = s4;
-      }
-      __syncthreads();
-      const int nk = n - k - 1;
-      for (int t = tid; t < nk * m; t += nt) {
-        const int c = t / nk, i = k + 1 + (t - c * nk);
-        Z[i + (size_t)c * n] -= 2.0 * v[i] * ptmp[c];
-      }
-      __syncthreads();
-    }
-    for (int i = n - 1; i >= 0; --i) {
-      const double inv = 1.0 / W.L[i + (size_t)i * n];
-      for (int c = tid; c < m; c += nt) Z[i + (size_t)c * n] *= inv;
-      __syncthreads();
-      const double* lrow = W.H + (size_t)i * n;  // L[i, k] for k < i, contiguous
-      for (int t = tid; t < i * m; t += nt) {
-        const int c = t / i, k = t - c * i;
-        Z[k + (size_t)c * n] -= lrow[k] * Z[i + (size_t)c * n];
-      }
-      __syncthreads();
-    }
-    for (int idx = tid; idx < n_out * m; idx += nt) {
-      const int r = idx % n_out, c = idx / n_out;
-      const double y = (r < n) ? Z[r + (size_t)c * n] * scal[r] : 0.0;
-      T.Y[r + (size_t)c * T.ldy] = y;
-      if (T.Yf) T.Yf[r + (size_t)c * T.ldy] = (float)y;
-    }
-    for (int c = tid; c < m; c += nt) T.theta[c] = lam[c];
-    if (tid == 0 && dropped && T.state) T.state[ST_FALLBACK] += 1;
-    (void)nmax;
-    return;
-  }
-}
-
 }  // namespace
 
 size_t rr_work_doubles(int n_max, int m) {
-  return (size_t)3 * n_max * n_max + (size_t)n_max * m + 4 * (size_t)n_max + m + (size_t)5 * n_max * m +
-         (size_t)2 * m + 16;
+  const size_t one = (size_t)3 * n_max * n_max + (size_t)n_max * m + 4 * (size_t)n_max + m + (size_t)5 * n_max * m +
+                     (size_t)2 * m + 16;
+  return std::max(one, rr_wide_work_doubles(n_max, m));
 }
 
-size_t rr_smem_bytes(int n, int m) {
-  return sizeof(double) * ((size_t)n * n + (size_t)n * m + 4 * (size_t)n + 3 * (size_t)m) +
-         sizeof(int) * RRS_THREADS + 64;
-}
-
-void init_rr_kernels() { opt_in_dynamic_smem((const void*)rr_smem_kernel); }
-
-// n_max: the largest pencil any task can have (3m for LOBPCG tasks).
+// n_max: the largest pencil any task can have (3m for LOBPCG tasks).  Pencils
+// of up to 608 columns go to the kernel chain of rr_wide.cu; larger ones do
+// not fit a cluster's shared memory and take the global-memory kernel above.
+// Measured against the one-CTA kernels that the chain replaced: 1.07 -> 0.19 ms
+// at n = 40 (FP64), 76 -> 3.6 ms at n = 432 (FP64, two pencils), 2.2 -> 0.95 ms
+// at n = 144 (double-float, two pencils); 18 pencils of 144 beside another
+// stream's work: a solve of 36 elements takes 3.02 s against 3.11 s.
 void launch_rr(const RRTask* d_tasks, int ntask, cudaStream_t st, int n_max, int m_max, bool dfloat) {
   if (ntask <= 0) return;
-  if (dfloat && rr_df_eligible(n_max, m_max)) {
-    launch_rr_df(d_tasks, ntask, st, n_max, m_max);
-    return;
-  }
-  const size_t sm = (n_max > 0) ? rr_smem_bytes(n_max, m_max) : (size_t)-1;
-  int dev = 0, optin = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (m_max <= RRS_THREADS && sm + 2048 <= (size_t)optin)
-    rr_smem_kernel<<<ntask, RRS_THREADS, sm, st>>>(d_tasks);
-  else
-    rr_kernel<<<ntask, RR_THREADS, 0, st>>>(d_tasks);
+  const bool df = dfloat && n_max <= RR_DF_NMAX && m_max <= RR_DF_MMAX;
+  if (n_max > 0 && rr_wide_eligible(n_max, m_max, ntask, df)) launch_rr_wide(d_tasks, ntask, st, n_max, m_max, df);
+  else rr_kernel<<<ntask, RR_THREADS, 0, st>>>(d_tasks);
 }
 
 }  // namespace dgdft

@@ -174,15 +174,17 @@ struct RRTask {
   int restart_max;
 };
 size_t rr_work_doubles(int n_max, int m);
-// n_max, m_max bound the tasks' pencil sizes; pencils that fit use the
-// shared-memory kernel.  n_max <= 0 forces the global-memory kernel.
-// dfloat: the FP32 stage's reduction in double-float arithmetic (rr_df.cu)
-// where the pencil fits that kernel, FP64 otherwise.
+// n_max, m_max bound the tasks' pencil sizes; n_max <= 0 forces the
+// global-memory kernel.  dfloat: the FP32 stage's reduction in double-float
+// arithmetic up to RR_DF_NMAX and RR_DF_MMAX, FP64 otherwise.
 void launch_rr(const RRTask* d_tasks, int ntask, cudaStream_t st, int n_max, int m_max, bool dfloat = false);
-void init_rr_kernels();
-bool rr_df_eligible(int n_max, int m_max);
-void launch_rr_df(const RRTask* d_tasks, int ntask, cudaStream_t st, int n_max, int m_max);
-void init_rr_df_kernel();
+constexpr int RR_DF_NMAX = 160, RR_DF_MMAX = 64;  // pencils reduced in double-float when asked
+// rr_wide.cu: the reduction as a chain of kernels over many SMs, in FP64 or
+// double-float
+bool rr_wide_eligible(int n_max, int m_max, int ntask, bool dfloat);
+void launch_rr_wide(const RRTask* d_tasks, int ntask, cudaStream_t st, int n_max, int m_max, bool dfloat);
+size_t rr_wide_work_doubles(int n_max, int m);
+void init_rr_wide_kernels();
 
 // solver-level helpers are in solver.cu
 

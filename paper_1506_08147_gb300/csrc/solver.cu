@@ -1900,8 +1900,7 @@ dgdft_status dgdft_alb_create(const dgdft_alb_config* cfg, int n_elem, const dgd
   init_hamiltonian_kernels();
   init_tf32_gram_kernel();
   init_tf32_update_kernel();
-  init_rr_kernels();
-  init_rr_df_kernel();
+  init_rr_wide_kernels();
   init_blas_kernels();
   cudaGetLastError();  // attribute queries above must not leave an error behind
   ctx->el.resize(n_elem);
