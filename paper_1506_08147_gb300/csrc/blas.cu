@@ -225,6 +225,11 @@ __global__ void __launch_bounds__(144) gram48_kernel(const ElemDev<float>* __res
 // thread reading 2 rows of a column as one 16-byte double2 (chunks of a
 // column swizzled by column group as there).  FP64 accumulation; the FP64
 // pipe bounds it, and 48-wide tiles avoid the 64-wide tiles' idle lanes.
+// Narrow blocks take only the ceil(m/4)^2 threads of one tile per row group:
+// the CTA's threads form up to eight groups that share a stage's rows and add
+// up at the end, so that no FP64 instruction works on columns past m (m = 16,
+// 4,096 rows: 1,420 us per launch with all threads on the 48-wide tile and two
+// chunks, 32 us with eight groups and launch_gram's shorter chunks).
 // grid: (npairs, nchunk, nel); block 144.
 constexpr int GKD = 16;  // rows per stage (doubles)
 
@@ -248,7 +253,11 @@ __global__ void __launch_bounds__(144) gram48d_kernel(const ElemDev<double>* __r
   const double* B = resolve(e, job.b[pair]);
   const int lda = ld_of(e, job.a[pair], job.ld_in, rows);
   const int ldb = ld_of(e, job.b[pair], job.ld_in, rows);
-  const int tx = threadIdx.x % 12, ty = threadIdx.x / 12;
+  // tile of td x td threads (4 x 4 outputs each), ngrp groups of them
+  const int td = (max(ca, cb) + 3) / 4;
+  const int ngrp = min(8, 144 / (td * td));
+  const int grp = threadIdx.x / (td * td), tt = threadIdx.x - grp * td * td;
+  const int tx = tt % td, ty = tt / td;
   const int k_beg = blockIdx.y * kchunk;
   const int k_end = min(rows, k_beg + kchunk);
   const bool vec = ((lda | ldb | k_beg) & 1) == 0 && ((((uintptr_t)A) | ((uintptr_t)B)) & 15) == 0;
@@ -294,8 +303,9 @@ __global__ void __launch_bounds__(144) gram48d_kernel(const ElemDev<double>* __r
     __syncthreads();
     const double* as = As[st & 1];
     const double* bs = Bs[st & 1];
+    if (grp < ngrp)
 #pragma unroll 2
-    for (int r = 0; r < GKD; r += 2) {
+    for (int r = 2 * grp; r < GKD; r += 2 * ngrp) {
       double2 a2[4], b2[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) a2[i] = *reinterpret_cast<const double2*>(as + g48d_off(ty * 4 + i, r));
@@ -307,6 +317,23 @@ __global__ void __launch_bounds__(144) gram48d_kernel(const ElemDev<double>* __r
         for (int j = 0; j < 4; ++j) acc[i][j] = fma(a2[i].y, b2[j].y, fma(a2[i].x, b2[j].x, acc[i][j]));
     }
     __syncthreads();
+  }
+  if (ngrp > 1) {
+    // the groups' sums, added in group order (a group holds at most 36 threads)
+    double* sums = &As[0][0];
+    for (int g = 1; g < ngrp; ++g) {
+      if (grp == g)
+#pragma unroll
+        for (int q = 0; q < 16; ++q) sums[q * (td * td) + tt] = acc[q >> 2][q & 3];
+      __syncthreads();
+      if (grp == 0)
+#pragma unroll
+        for (int q = 0; q < 16; ++q) acc[q >> 2][q & 3] += sums[q * (td * td) + tt];
+      __syncthreads();
+    }
+    if (grp > 0) return;
+  } else if (grp > 0) {
+    return;
   }
   double* out = partial + blockIdx.z * pstride + ((size_t)blockIdx.y * gridDim.x + pair) * (TILE * TILE);
 #pragma unroll
@@ -1093,8 +1120,10 @@ void launch_gram(const Batch<real>& b, const GramJob<real>& job, double* partial
   const int rows = job.rows > 0 ? job.rows : s.max_ng;
   const int tiles_a = (ca + TILE - 1) / TILE, tiles_b = (cb + TILE - 1) / TILE;
   const int ny = job.npairs * tiles_a * tiles_b;
-  // per-element partial storage: nchunk * ny tiles
+  // per-element partial storage: nchunk * ny tiles.  Chunks of 2,048 rows, or
+  // of as few as 128 while the grid would not give every SM two CTAs
   int kchunk = 2048;
+  while (kchunk > 128 && (size_t)((rows + kchunk - 1) / kchunk) * ny * s.nel < 304) kchunk /= 2;
   int nchunk = (rows + kchunk - 1) / kchunk;
   while ((size_t)nchunk * ny * TILE * TILE * s.nel > partial_cap && kchunk < (1 << 30)) {
     kchunk *= 2;

@@ -86,6 +86,13 @@ void launch_h_pass(const Batch<real>& b, int pass, BRef<real> src, BRef<real> ds
 // chunks; FP64 partial sums are reduced in a fixed order.
 enum { OUT_GRAM_A = 0, OUT_GRAM_B = 1, OUT_GXW = 2, OUT_PTR = 3 };
 constexpr int MAX_PAIRS = 12;
+// Gram partials of one element: 12 products of m x m in 64 x 64 tiles per row
+// chunk, chunks of 2,048 rows but room for 16 of them (shorter ones where
+// there are few)
+inline size_t gram_partial_doubles(size_t ng, size_t m) {
+  const size_t chunks = (ng + 2047) / 2048, tiles = (m + 63) / 64;
+  return (chunks < 16 ? 16 : chunks) * 12 * tiles * tiles * 4096;
+}
 template <class real> struct GramJob {
   int npairs = 0;
   BRef<real> a[MAX_PAIRS], b[MAX_PAIRS];
@@ -185,6 +192,14 @@ bool rr_wide_eligible(int n_max, int m_max, int ntask, bool dfloat);
 void launch_rr_wide(const RRTask* d_tasks, int ntask, cudaStream_t st, int n_max, int m_max, bool dfloat);
 size_t rr_wide_work_doubles(int n_max, int m);
 void init_rr_wide_kernels();
+void launch_rr_standard(const RRTask* d_task, int n, int m, cudaStream_t st);
+// eigh.cu: the lowest m eigenpairs (theta ascending, orthonormal columns Y) of
+// one dense symmetric FP64 matrix.  h: an RR_FIXED task (n_fixed = n <= 4096,
+// m, Y, ldy, theta, work of eigh_work_doubles(n, m)), d_task its copy on the
+// device; the matrix is put at eigh_matrix(h), n x n, and overwritten.
+size_t eigh_work_doubles(int n, int m);
+double* eigh_matrix(const RRTask& h);
+cudaError_t launch_eigh(const RRTask& h, const RRTask* d_task, cudaStream_t st);
 
 // solver-level helpers are in solver.cu
 

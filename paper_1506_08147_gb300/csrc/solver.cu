@@ -441,8 +441,7 @@ template <class real> struct Wave {
     // in double-float arithmetic; the plain FP64 solver stays on the FP64 pipe
     s.dfloat = std::is_same<real, double>::value && ctx->cfg.precision == DGDFT_PREC_MIXED;
     rnchunk = nchunk_rows(s.max_ng);
-    const size_t tiles = ((s.max_m + 63) / 64) * ((s.max_m + 63) / 64);
-    const size_t pcap = (size_t)nel * ((s.max_ng + 2047) / 2048) * 12 * tiles * 4096;
+    const size_t pcap = (size_t)nel * gram_partial_doubles(s.max_ng, s.max_m);
     size_t total = 0;
     for (int id : ids) {
       total += elem_bytes<real>(ctx->el[id]);
@@ -1798,8 +1797,7 @@ dgdft_status plan_waves(dgdft_alb_ctx* ctx, std::vector<std::vector<int>>& waves
     // plus the element's share of the wave-level buffers (Gram partials and
     // residual partial sums, sized here by the element itself)
     const size_t m = (size_t)eh.d.n_compute, ng = (size_t)eh.ng();
-    const size_t shared = sizeof(double) * (((ng + 2047) / 2048) * 12 * ((m + 63) / 64) * ((m + 63) / 64) * 4096 +
-                                            m * (size_t)nchunk_rows((int)ng) * 4);
+    const size_t shared = sizeof(double) * (gram_partial_doubles(ng, m) + m * (size_t)nchunk_rows((int)ng) * 4);
     size_t b = elem_bytes<double>(eh) + shared;
     if (ctx->cfg.precision == DGDFT_PREC_MIXED) b += elem_bytes<float>(eh) + shared;
     if (b > cap) return ctx->fail(DGDFT_ENOMEM, "one element exceeds the device-memory budget");
@@ -2204,7 +2202,7 @@ dgdft_status gram_t(dgdft_alb_ctx* ctx, int ng, int p, int q, const double* u, c
   ElemDev<real>* de = nullptr;
   int* dstate = nullptr;
   const size_t tiles = ((p + 63) / 64) * ((q + 63) / 64);
-  const size_t pcap = ((size_t)(ng + 2047) / 2048) * tiles * 4096;
+  const size_t pcap = std::max<size_t>(16, ((size_t)ng + 2047) / 2048) * tiles * 4096;
   CK(cudaMalloc(&du, sizeof(real) * (size_t)ng * p));
   CK(cudaMalloc(&dv, sizeof(real) * (size_t)ng * q));
   CK(cudaMalloc(&dc, sizeof(double) * (size_t)p * q));
