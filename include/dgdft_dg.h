@@ -124,9 +124,8 @@ dgdft_status dgdft_dg_lgl_basis(dgdft_dg* dg, int elem, const double* z, int z_o
 /* Density (Eq. density) by dense diagonalisation of the assembled H^DG (the
  * DIAG route of Sec. II.B, for small systems): the lowest n_occ eigenpairs
  * of H^DG c = lambda c (the basis is orthonormal, so a standard problem) by
- * an FP64 one-sided Jacobi eigensolver over the whole GPU (sweeps until no
- * pair of columns has a cosine above sqrt(n) 1e-15, at most 40; DGDFT_ENOTCONV
- * beyond), then rho(x) = sum_{i < n_occ}
+ * FP64 Householder tridiagonalisation and inverse iteration over the whole
+ * GPU (DGDFT_ENOTCONV when an eigenvalue is not finite), then rho(x) = sum_{i < n_occ}
  * |psi_i(x)|^2 with psi_i = sum_{K,j} c_{i;K,j} phi_{K,j}, one electron per
  * state as Eq. density is written, on every element's LGL grid.  z: the same
  * columns as the last assemble (z_on_device as there; the basis is rebuilt
@@ -137,7 +136,8 @@ dgdft_status dgdft_dg_lgl_basis(dgdft_dg* dg, int elem, const double* z, int z_o
 dgdft_status dgdft_dg_density(dgdft_dg* dg, const double* const* z, int z_on_device, int n_occ, double* eig,
                               double* rho, int on_device);
 
-/* Sweeps of the Jacobi eigensolver in the last dgdft_dg_density (host int). */
+/* Sweeps over the matrix that the eigensolver of the last dgdft_dg_density took
+ * (host int): 1, as it is a direct solver; 0 before any density. */
 dgdft_status dgdft_dg_density_info(dgdft_dg* dg, int* sweeps);
 
 /* Kernel time of the last assembly per stage (CUDA events on the stream):

@@ -582,7 +582,7 @@ class DG:
         return phi
 
     def dgdft_dg_density_info(self):
-        """Sweeps of the Jacobi eigensolver in the last density call."""
+        """Sweeps over the matrix that the eigensolver of the last density call took."""
         n = C.c_int()
         self._check(self.lib.dgdft_dg_density_info(self.h, C.byref(n)), "density_info")
         return n.value
