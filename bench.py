@@ -265,7 +265,7 @@ def dg_measure(B, dom, blocks, stream, steps, warmup, cap_bytes=0, dfloat=False,
             "sweeps": d.dgdft_dg_density_info(),
             "eigensolve_ms": round(dens_stage["density_eigensolve"], 2),
             "evaluation_ms": round(dens_stage["density_evaluation"], 2),
-            "eigensolver": "FP64 one-sided Jacobi, one cooperative kernel over all SMs"}
+            "eigensolver": "FP64 Householder tridiagonalisation and inverse iteration, a cooperative kernel over all SMs"}
     del rho
     d.close()
     out["density"] = dens

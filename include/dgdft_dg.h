@@ -25,7 +25,7 @@
  *     (d_d u_a + d_d u_b) / 2; with one element along d the face joins the
  *     element to itself across the periodic boundary.
  *
- * Arithmetic: FP64 by default, double-float pairs as an option (arith).
+ * Arithmetic: FP64 (contractions to 2^-54 of the largest entry of a row).
  * All compute runs on the GPU on the stream of the configuration; there is
  * no CPU path.
  */
@@ -59,14 +59,13 @@ typedef struct {
   size_t hbm_cap_bytes; /* bound on the per-batch scratch (0 = a quarter of
                            the free device memory); elements are processed
                            in batches that fit it                          */
-  int arith;            /* contractions (interpolation, orthonormalisation,
-                           differentiation, Gram products): 0 = FP64;
-                           1 = double-float pairs on the FP32 pipes
-                           (~2^-48 relative per operation, ~3x faster).
-                           With nearly dependent columns (mass-matrix
-                           condition kappa) both forms lose about
-                           kappa^(1/2) of their unit in the basis's weak
-                           directions, double-float from its larger unit */
+  int arith;            /* 0 = FP64, 1 = double-float pairs (2^-48 relative per
+                           operation) suffice for the contractions.  Both run
+                           the same kernels: FP64 products on the tensor cores
+                           by exact digit splitting, faster than pairs on the
+                           FP32 pipes.  With nearly dependent columns
+                           (mass-matrix condition kappa) the basis's weak
+                           directions lose about kappa^(1/2) of the unit    */
 } dgdft_dg_config;
 
 /* Validate the configuration, build the LGL, differentiation and
@@ -103,7 +102,9 @@ dgdft_status dgdft_dg_set_projectors(dgdft_dg* dg, int elem, int n_p, const int*
  * only, not retained).  Results stay on the device until dgdft_dg_get_row.
  * DGDFT_EINVAL on a NULL pointer; DGDFT_ENOTCONV when a mass matrix is not
  * positive definite (columns linearly dependent on E_K; the element is named
- * in dgdft_dg_last_error); DGDFT_ECUDA on a CUDA error.                     */
+ * in dgdft_dg_last_error); DGDFT_ETIMEOUT when a bounded device wait ran out
+ * (also from dgdft_dg_lgl_basis and dgdft_dg_density); DGDFT_ECUDA on a CUDA
+ * error.                                                                    */
 dgdft_status dgdft_dg_assemble(dgdft_dg* dg, const double* const* z, int on_device);
 
 /* The distinct elements of the 3 x 3 x 3 periodic neighbourhood of `elem`,

@@ -1,7 +1,8 @@
 // DG Hamiltonian assembly from the adaptive local basis (Eq. DGHamiltonian;
 // Sec. II.B, "Construction of the DG Hamiltonian").
 //
-// Per batch of elements, FP64 throughout:
+// Per batch of elements, FP64 throughout (the axis passes and Gram products on
+// the tensor cores by exact digit splitting, dg_tensor.cu):
 //   1. interpolation of the J columns from Q_K's uniform grid to E_K's LGL
 //      grid: three passes of a small dense matrix applied along one axis
 //      (the real trigonometric interpolant over Q_K, sampled at the nodes);
@@ -21,8 +22,8 @@
 //   7. every block H_{K,K'} summed from its volume, KB and face terms.
 // Density (Eq. density, the DIAG route for small systems): H^DG scattered
 // into a dense matrix, its eigenpairs by tridiagonalisation over the whole GPU
-// (eigh.cu), the density matrix blocks P_K = Y_K Y_K^T of the lowest n_occ, and rho = sum_jj' phi_j P_K,jj' phi_j'
-// on the LGL grids.
+// (eigh.cu), the density matrix blocks P_K = Y_K Y_K^T of the lowest n_occ, and
+// rho = sum_jj' phi_j P_K,jj' phi_j' on the LGL grids.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -35,135 +36,34 @@
 #include <vector>
 
 #include "../../include/dgdft_dg.h"
-#include "dfloat.cuh"
+#include "dg_tensor.h"
 #include "internal.h"
 
 namespace {
 
-constexpr int AX_THREADS = 256;
-constexpr int AX_TC = 64;                      // columns per CTA tile
-constexpr int AX_LD = AX_TC + 1;               // odd stride: conflict-free column walks
-constexpr int AX_NR = AX_THREADS / AX_TC;      // row groups
-constexpr int AX_MAXR = 32;                    // output rows per thread: n_out <= 128
-constexpr int MAX_NL = AX_MAXR * AX_NR;
+constexpr int MAX_NL = 128;
 constexpr int MAX_J = 128;
-
-constexpr int GR_R = 16;                       // staged points per step
-constexpr int GR_CH = 2048;                    // points per split-K chunk
 
 constexpr double PI = 3.14159265358979323846;
 
-// Arithmetic of the contractions: FP64, or double-float pairs (FP32 h + l,
-// ~2^-48 relative per operation, on the FP32 pipes).
-using dgdft::dfl;
+using dgdft::axis_image_bytes;
+using dgdft::gram_tensor_chunk;
+using dgdft::gram_tensor_items;
+using dgdft::launch_axis_tensor;
+using dgdft::launch_gram_tensor;
+using dgdft::TGramTask;
 using dgdft::eigh_matrix;
 using dgdft::eigh_work_doubles;
 using dgdft::launch_eigh;
 using dgdft::RRTask;
 using dgdft::RR_FIXED;
-__device__ __forceinline__ double to_t(double v, double*) { return v; }
-__device__ __forceinline__ dfl to_t(double v, dfl*) { return dgdft::dfl_of(v); }
-__device__ __forceinline__ double fma_t(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ dfl fma_t(dfl a, dfl b, dfl c) { return dgdft::dfl_fma(a, b, c); }
-__device__ __forceinline__ double val_t(double a) { return a; }
-__device__ __forceinline__ double val_t(dfl a) { return dgdft::dfl_val(a); }
-template <class T> __device__ __forceinline__ T zero_t() { return to_t(0.0, (T*)nullptr); }
 
 // ------------------------------------------------------------------ kernels
 
-// One pass of a small dense matrix A (n_out x n_in, row-major; element e uses
-// A + e * a_stride) along one axis of every element's array viewed as
-// [O][n_in][S]: out[o][r][s] = sum_i A[r][i] in[o][i][s].  FAST (S == 1): a
-// tile is 64 consecutive lines, staged transposed so loads and stores stay
-// coalesced; otherwise a tile is 64 consecutive (o, s) columns, s fastest.
-// Each thread owns R output rows of one column (R >= n_out / AX_NR, a
-// compile-time count, so no FP64 instruction issues for rows that do not
-// exist beyond the last group of AX_NR).
-struct AxisJob {
-  const double* const* in;
-  double* const* out;
-  const double* A;
-  long long a_stride;
-  int n_in, n_out, S;
-  long long O;
-};
-
-template <bool FAST, int R, class T>
-__global__ void __launch_bounds__(AX_THREADS) dg_axis_kernel(AxisJob jb) {
-  extern __shared__ double sm[];
-  const int nin = jb.n_in, nout = jb.n_out, S = jb.S;
-  T* As = reinterpret_cast<T*>(sm);
-  T* Xs = As + nout * nin;
-  const double* __restrict__ in = jb.in[blockIdx.y];
-  double* __restrict__ out = jb.out[blockIdx.y];
-  const double* __restrict__ A = jb.A + blockIdx.y * jb.a_stride;
-  const int t = threadIdx.x;
-  for (int i = t; i < nout * nin; i += AX_THREADS) As[i] = to_t(A[i], (T*)nullptr);
-  const long long ncols_total = FAST ? jb.O : jb.O * (long long)S;
-  const long long g0 = (long long)blockIdx.x * AX_TC;
-  const int ncol = (int)min((long long)AX_TC, ncols_total - g0);
-  if (FAST) {
-    const double* src = in + g0 * nin;
-    for (int q = t; q < ncol * nin; q += AX_THREADS) {
-      const int c = q / nin, i = q - c * nin;
-      Xs[i * AX_LD + c] = to_t(src[q], (T*)nullptr);
-    }
-  } else {
-    for (int q = t; q < nin * AX_TC; q += AX_THREADS) {
-      const int i = q / AX_TC, c = q - i * AX_TC;
-      double v = 0.0;
-      if (c < ncol) {
-        const long long g = g0 + c, o = g / S, s = g - o * S;
-        v = in[(o * nin + i) * S + s];
-      }
-      Xs[i * AX_LD + c] = to_t(v, (T*)nullptr);
-    }
-  }
-  __syncthreads();
-  const int c = t % AX_TC, r = t / AX_TC;
-  // rows r, r + AX_NR, ...: the last ones may not exist (row >= nout); their
-  // matrix row is clamped to a valid one and the result is not stored
-  int arow[R];
-#pragma unroll
-  for (int k = 0; k < R; ++k) arow[k] = min(r + k * AX_NR, nout - 1) * nin;
-  T acc[R];
-#pragma unroll
-  for (int k = 0; k < R; ++k) acc[k] = zero_t<T>();
-  for (int i = 0; i < nin; ++i) {
-    const T x = Xs[i * AX_LD + c];
-#pragma unroll
-    for (int k = 0; k < R; ++k) acc[k] = fma_t(As[arow[k] + i], x, acc[k]);
-  }
-  if (FAST) {
-    __syncthreads();
-    double* Xd = reinterpret_cast<double*>(Xs);  // the tile again, as doubles
-#pragma unroll
-    for (int k = 0; k < R; ++k) {
-      const int row = r + k * AX_NR;
-      if (row < nout) Xd[row * AX_LD + c] = val_t(acc[k]);
-    }
-    __syncthreads();
-    double* dst = out + g0 * nout;
-    for (int q = t; q < ncol * nout; q += AX_THREADS) {
-      const int cc = q / nout, i = q - cc * nout;
-      dst[q] = Xd[i * AX_LD + cc];
-    }
-  } else if (c < ncol) {
-    const long long g = g0 + c, o = g / S, s = g - o * S;
-#pragma unroll
-    for (int k = 0; k < R; ++k) {
-      const int row = r + k * AX_NR;
-      if (row < nout) out[(o * nout + row) * S + s] = val_t(acc[k]);
-    }
-  }
-}
-
 // Weighted Gram products C = X^T diag(w v) Y over n points (X, Y column-major
-// with leading dimensions ldx, ldy), split into chunks of GR_CH points whose
-// partial J1 x J2 sums are added in a fixed order by dg_gram_reduce_kernel.
-// Each thread owns a 2 x 2 output tile; tiles are numbered densely (row-major,
-// or the upper triangle ti <= tj when sym: X = Y, the lower half mirrored by
-// the reduction), 256 per CTA, grid.z over groups of 256 tiles.
+// with leading dimensions ldx, ldy), split into chunks whose partial J1 x J2
+// sums are added in a fixed order by dg_gram_reduce_kernel.  sym: X = Y, the
+// lower half is the mirrored upper one.
 struct GramTask {
   const double* X;
   const double* Y;
@@ -174,90 +74,12 @@ struct GramTask {
   int n, ldx, ldy, J1, J2, nchunk, sym;
 };
 
-__device__ __forceinline__ void gram_tile_of(int t, int nt, int sym, int* ti, int* tj) {
-  if (!sym) {
-    *ti = t / nt;
-    *tj = t - *ti * nt;
-    return;
-  }
-  // upper triangle, row by row: row i holds nt - i tiles
-  int i = 0, base = 0;
-  while (t >= base + (nt - i)) {
-    base += nt - i;
-    ++i;
-  }
-  *ti = i;
-  *tj = i + (t - base);
-}
-
-template <class T>
-__global__ void __launch_bounds__(256) dg_gram_kernel(const GramTask* __restrict__ tasks,
-                                                      double* __restrict__ partial) {
-  __shared__ T Xs[GR_R][MAX_J + 2];
-  __shared__ T Ys[GR_R][MAX_J + 2];
-  const GramTask Tk = tasks[blockIdx.y];
-  const int chunk = blockIdx.x;
-  if (chunk >= Tk.nchunk) return;
-  const int nti = (Tk.J1 + 1) / 2, ntj = (Tk.J2 + 1) / 2;
-  const int ntiles = Tk.sym ? nti * (nti + 1) / 2 : nti * ntj;
-  const int tile0 = blockIdx.z * 256;
-  if (tile0 >= ntiles) return;
-  const int mytile = tile0 + threadIdx.x;
-  int ti = 0, tj = 0;
-  const bool active = mytile < ntiles;
-  if (active) gram_tile_of(mytile, Tk.sym ? nti : ntj, Tk.sym, &ti, &tj);
-  const int i0 = 2 * ti, j0 = 2 * tj;
-  const int p0 = chunk * GR_CH, p1 = min(Tk.n, p0 + GR_CH);
-  T acc00 = zero_t<T>(), acc01 = zero_t<T>(), acc10 = zero_t<T>(), acc11 = zero_t<T>();
-  const int J1p = (Tk.J1 + 1) & ~1, J2p = (Tk.J2 + 1) & ~1;
-  for (int p = p0; p < p1; p += GR_R) {
-    for (int q = threadIdx.x; q < GR_R * J1p; q += 256) {
-      const int col = q / GR_R, rr = q - col * GR_R, pt = p + rr;
-      double xv = 0.0;
-      if (pt < p1 && col < Tk.J1) {
-        double wt = Tk.w[pt];
-        if (Tk.v) wt *= Tk.v[pt];
-        xv = Tk.X[(size_t)col * Tk.ldx + pt] * wt;
-      }
-      Xs[rr][col] = to_t(xv, (T*)nullptr);
-    }
-    for (int q = threadIdx.x; q < GR_R * J2p; q += 256) {
-      const int col = q / GR_R, rr = q - col * GR_R, pt = p + rr;
-      Ys[rr][col] = to_t((pt < p1 && col < Tk.J2) ? Tk.Y[(size_t)col * Tk.ldy + pt] : 0.0, (T*)nullptr);
-    }
-    __syncthreads();
-    if (active) {
-#pragma unroll
-      for (int rr = 0; rr < GR_R; ++rr) {
-        const T a0 = Xs[rr][i0], a1 = Xs[rr][i0 + 1];
-        const T b0 = Ys[rr][j0], b1 = Ys[rr][j0 + 1];
-        acc00 = fma_t(a0, b0, acc00);
-        acc01 = fma_t(a0, b1, acc01);
-        acc10 = fma_t(a1, b0, acc10);
-        acc11 = fma_t(a1, b1, acc11);
-      }
-    }
-    __syncthreads();
-  }
-  if (!active) return;
-  double* dst = partial + Tk.part + (size_t)chunk * Tk.J1 * Tk.J2;
-  const double v[2][2] = {{val_t(acc00), val_t(acc01)}, {val_t(acc10), val_t(acc11)}};
-#pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int b = 0; b < 2; ++b) {
-      const int ii = i0 + a, jj = j0 + b;
-      if (ii < Tk.J1 && jj < Tk.J2) dst[(size_t)ii * Tk.J2 + jj] = v[a][b];
-    }
-}
-
 __global__ void dg_gram_reduce_kernel(const GramTask* __restrict__ tasks, const double* __restrict__ partial) {
   const GramTask T = tasks[blockIdx.y];
   const int n = T.J1 * T.J2;
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
     int i = q / T.J2, j = q - (q / T.J2) * T.J2;
-    // symmetric tasks hold the tiles with i/2 <= j/2 only
-    if (T.sym && i / 2 > j / 2) {
+    if (T.sym && i > j) {
       const int t = i;
       i = j;
       j = t;
@@ -339,15 +161,19 @@ __global__ void dg_kb_kernel(KbJob jb) {
 
 // Cholesky M~ = L L^T of every element's mass matrix (in shared memory) and
 // the lower triangular L^-1 (written column by column to global memory, each
-// column by one thread), one CTA per element.
+// column by one thread), one CTA per element.  shift: the binary exponents of
+// the columns' norms.
 __global__ void __launch_bounds__(256) dg_chol_kernel(const double* __restrict__ mass, long long mass_stride,
-                                                      double* __restrict__ linv, int J, int* __restrict__ bad) {
+                                                      double* __restrict__ linv, int J, int* __restrict__ bad,
+                                                      int* __restrict__ shift) {
   extern __shared__ double Ls[];  // J x J
   const int e = blockIdx.x, t = threadIdx.x;
   const double* M = mass + (size_t)e * mass_stride;
   for (int q = t; q < J * J; q += blockDim.x) Ls[q] = M[q];
   __shared__ int fail;
   if (t == 0) fail = 0;
+  for (int q = t; q < J; q += blockDim.x)
+    shift[(size_t)e * J + q] = (((__double2hiint(M[(size_t)q * J + q]) >> 20) & 0x7ff) - 1023) >> 1;
   __syncthreads();
   for (int k = 0; k < J; ++k) {
     if (t == 0) {
@@ -559,7 +385,7 @@ struct dgdft_dg {
   std::vector<double> xr[3], wr[3], local[3], w1[3];
   double le[3]{}, e_off[3]{};
   // device tables
-  double *d_I[3]{}, *d_D[3]{}, *d_w = nullptr, *d_wf[3]{};
+  double *d_I[3]{}, *d_D[3]{}, *d_w = nullptr, *d_sw = nullptr, *d_wf[3]{};
   // inputs
   double* d_v = nullptr;  // nel x nL
   std::vector<double> gamma;
@@ -586,6 +412,10 @@ struct dgdft_dg {
   int density_sweeps = 0;  // sweeps of the eigensolver in the last density
   double* d_eig = nullptr;  // its work, kept between calls
   size_t eig_cap = 0;
+  // digit images of an axis pass, Gram task lists: kept, grown when needed
+  void *d_img = nullptr, *d_tasks = nullptr, *d_shift = nullptr;
+  size_t img_cap = 0, tasks_cap = 0, shift_cap = 0;
+  int* d_terr = nullptr;  // set by a tensor-core kernel whose wait ran out
   int launches = 0;
   // batch scratch
   int batch = 0;
@@ -633,71 +463,64 @@ template <class T> bool upload(dgdft_dg* dg, T** p, const std::vector<T>& h) {
          cudaStreamSynchronize(dg->st) == cudaSuccess;
 }
 
-size_t axis_smem(int nin, int nout) {
-  return sizeof(double) * ((size_t)nout * nin + (size_t)std::max(nin, nout) * AX_LD);
+// size of a pass's matrix and of 65 of its lines: the limit on the grids
+size_t axis_size(int nin, int nout) {
+  return sizeof(double) * ((size_t)nout * nin + (size_t)std::max(nin, nout) * 65);
 }
 
-template <bool FAST, int R>
-void launch_axis_r(dgdft_dg* dg, const AxisJob& jb, unsigned tiles, int nelem, size_t sm) {
-  if (dg->cfg.arith)
-    dg_axis_kernel<FAST, R, dfl><<<dim3(tiles, nelem), AX_THREADS, sm, dg->st>>>(jb);
-  else
-    dg_axis_kernel<FAST, R, double><<<dim3(tiles, nelem), AX_THREADS, sm, dg->st>>>(jb);
-}
-
-template <bool FAST>
-void launch_axis_fast(dgdft_dg* dg, const AxisJob& jb, unsigned tiles, int nelem, size_t sm) {
-  const int need = (jb.n_out + AX_NR - 1) / AX_NR;
-  if (need <= 4) launch_axis_r<FAST, 4>(dg, jb, tiles, nelem, sm);
-  else if (need <= 8) launch_axis_r<FAST, 8>(dg, jb, tiles, nelem, sm);
-  else if (need <= 12) launch_axis_r<FAST, 12>(dg, jb, tiles, nelem, sm);
-  else if (need <= 16) launch_axis_r<FAST, 16>(dg, jb, tiles, nelem, sm);
-  else if (need <= 20) launch_axis_r<FAST, 20>(dg, jb, tiles, nelem, sm);
-  else if (need <= 24) launch_axis_r<FAST, 24>(dg, jb, tiles, nelem, sm);
-  else launch_axis_r<FAST, 32>(dg, jb, tiles, nelem, sm);
-}
-
-template <bool FAST, int R> bool set_smem_r(int bytes) {
-  return cudaFuncSetAttribute(dg_axis_kernel<FAST, R, double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              bytes) == cudaSuccess &&
-         cudaFuncSetAttribute(dg_axis_kernel<FAST, R, dfl>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) ==
-             cudaSuccess;
-}
-
-template <bool FAST> bool set_axis_smem(int bytes) {
-  return set_smem_r<FAST, 4>(bytes) && set_smem_r<FAST, 8>(bytes) && set_smem_r<FAST, 12>(bytes) &&
-         set_smem_r<FAST, 16>(bytes) && set_smem_r<FAST, 20>(bytes) && set_smem_r<FAST, 24>(bytes) &&
-         set_smem_r<FAST, 32>(bytes);
+// device scratch that a handle keeps and grows
+bool keep_bytes(dgdft_dg* dg, void** p, size_t* cap, size_t bytes) {
+  if (bytes <= *cap) return true;
+  cudaFree(*p);
+  *p = nullptr;
+  *cap = 0;
+  if (cudaMalloc(p, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    *p = nullptr;
+    dg->err = "scratch: out of memory";
+    return false;
+  }
+  *cap = bytes;
+  return true;
 }
 
 // A (n_out x n_in) along one axis of nelem arrays [O][n_in][S]; element e
 // uses A + e * a_stride.
 bool launch_axis(dgdft_dg* dg, const double* const* d_in, double* const* d_out, int nelem, const double* A,
-                 int nin, int nout, int S, long long O, long long a_stride = 0) {
-  AxisJob jb{d_in, d_out, A, a_stride, nin, nout, S, O};
-  const long long cols = (S == 1) ? O : O * S;
-  const unsigned tiles = (unsigned)((cols + AX_TC - 1) / AX_TC);
-  const size_t sm = axis_smem(nin, nout);
-  if (S == 1)
-    launch_axis_fast<true>(dg, jb, tiles, nelem, sm);
-  else
-    launch_axis_fast<false>(dg, jb, tiles, nelem, sm);
-  ++dg->launches;
-  return cuda_ok(dg, cudaGetLastError(), "axis kernel");
+                 int nin, int nout, int S, long long O, long long a_stride = 0,
+                 const int* shift = nullptr) {
+  if (!keep_bytes(dg, &dg->d_img, &dg->img_cap, axis_image_bytes(nin, nout, a_stride ? nelem : 1))) return false;
+  dg->launches += 2;
+  return cuda_ok(dg, launch_axis_tensor(d_in, d_out, nelem, A, a_stride, nin, nout, S, O, shift, dg->d_img, dg->d_terr, dg->st),
+                 "axis kernel");
 }
 
 bool run_grams(dgdft_dg* dg, std::vector<GramTask>& tasks) {
   if (tasks.empty()) return true;
+  const int nt = (int)tasks.size();
   long long part = 0;
-  int maxc = 0, maxJ1 = 0, maxJ2 = 0;
-  for (GramTask& t : tasks) {
-    t.nchunk = (t.n + GR_CH - 1) / GR_CH;
+  int maxJ1 = 0, maxJ2 = 0, nexp = 0;
+  std::vector<TGramTask> tt(nt);
+  for (int i = 0; i < nt; ++i) {
+    GramTask& t = tasks[i];
+    const int chunk = gram_tensor_chunk(t.n);
+    t.nchunk = (t.n + chunk - 1) / chunk;
     t.part = part;
+    tt[i] = TGramTask{t.X, t.Y, t.w, t.v, part, t.n, t.ldx, t.ldy, t.J1, t.J2, chunk, nexp, 0};
     part += (long long)t.nchunk * t.J1 * t.J2;
-    maxc = std::max(maxc, t.nchunk);
+    nexp += t.J1 + t.J2;
     maxJ1 = std::max(maxJ1, t.J1);
     maxJ2 = std::max(maxJ2, t.J2);
   }
+  // volume products without a second factor: (sqrt(w) X)^T (sqrt(w) X), split once
+  if (maxJ1 == maxJ2 && maxJ2 <= 64)
+    for (int i = 0; i < nt; ++i)
+      if (tasks[i].sym && !tt[i].v && tt[i].w == dg->d_w && tt[i].X == tt[i].Y) {
+        tt[i].w = dg->d_sw;
+        tt[i].sym = 1;
+      }
+  std::vector<int> items;
+  gram_tensor_items(tt.data(), nt, items);
   if ((size_t)part > dg->part_cap) {
     cudaFree(dg->d_part);
     dg->d_part = nullptr;
@@ -708,28 +531,41 @@ bool run_grams(dgdft_dg* dg, std::vector<GramTask>& tasks) {
     }
     dg->part_cap = (size_t)part;
   }
-  GramTask* d_t = nullptr;
-  std::vector<GramTask> h(tasks);
-  if (!dmalloc(&d_t, h.size())) {
-    dg->err = "Gram tasks: out of memory";
-    return false;
-  }
-  bool ok = cuda_ok(dg, cudaMemcpyAsync(d_t, h.data(), h.size() * sizeof(GramTask), cudaMemcpyHostToDevice, dg->st),
-                    "Gram tasks");
-  const int ntiles = ((maxJ1 + 1) / 2) * ((maxJ2 + 1) / 2);
+  // both task lists, the items and the exponents in one kept buffer
+  const size_t b0 = nt * sizeof(GramTask), b1 = b0 + nt * sizeof(TGramTask), b2 = b1 + items.size() * sizeof(int);
+  if (!keep_bytes(dg, &dg->d_tasks, &dg->tasks_cap, b2 + nexp * sizeof(int))) return false;
+  std::vector<char> h(b2);
+  std::memcpy(h.data(), tasks.data(), b0);
+  std::memcpy(h.data() + b0, tt.data(), b1 - b0);
+  std::memcpy(h.data() + b1, items.data(), b2 - b1);
+  char* d = static_cast<char*>(dg->d_tasks);
+  bool ok = cuda_ok(dg, cudaMemcpyAsync(d, h.data(), b2, cudaMemcpyHostToDevice, dg->st), "Gram tasks");
   if (ok) {
-    const dim3 grid(maxc, (unsigned)h.size(), (ntiles + 255) / 256);
-    if (dg->cfg.arith)
-      dg_gram_kernel<dfl><<<grid, 256, 0, dg->st>>>(d_t, dg->d_part);
-    else
-      dg_gram_kernel<double><<<grid, 256, 0, dg->st>>>(d_t, dg->d_part);
-    dg_gram_reduce_kernel<<<dim3(std::max(1, (maxJ1 * maxJ2 + 255) / 256), (unsigned)h.size()), 256, 0, dg->st>>>(
-        d_t, dg->d_part);
-    dg->launches += 2;
-    ok = cuda_ok(dg, cudaGetLastError(), "Gram kernel") && cuda_ok(dg, cudaStreamSynchronize(dg->st), "Gram kernel");
+    ok = cuda_ok(dg,
+                 launch_gram_tensor(reinterpret_cast<TGramTask*>(d + b0), nt, reinterpret_cast<int*>(d + b1),
+                                    (int)items.size() / 3, maxJ1, maxJ2, reinterpret_cast<int*>(d + b2), dg->d_part,
+                                    dg->d_terr, dg->st),
+                 "Gram kernel");
+    dg_gram_reduce_kernel<<<dim3(std::max(1, (maxJ1 * maxJ2 + 255) / 256), (unsigned)nt), 256, 0, dg->st>>>(
+        reinterpret_cast<GramTask*>(d), dg->d_part);
+    dg->launches += 3;
+    ok = ok && cuda_ok(dg, cudaGetLastError(), "Gram kernel") &&
+         cuda_ok(dg, cudaStreamSynchronize(dg->st), "Gram kernel");
   }
-  cudaFree(d_t);
   return ok;
+}
+
+// false (and a message) when a bounded wait of the tensor-core kernels ran out
+// since the last check
+bool tensor_waits_ok(dgdft_dg* dg) {
+  int h = 0;
+  if (!cuda_ok(dg, cudaMemcpyAsync(&h, dg->d_terr, sizeof(int), cudaMemcpyDeviceToHost, dg->st), "status") ||
+      !cuda_ok(dg, cudaStreamSynchronize(dg->st), "status"))
+    return false;
+  if (!h) return true;
+  cudaMemsetAsync(dg->d_terr, 0, sizeof(int), dg->st);
+  dg->err = "a bounded device wait ran out";
+  return false;
 }
 
 struct Timer {
@@ -836,7 +672,9 @@ bool ortho_batch(dgdft_dg* dg, int nb, double* mass, long long mass_stride, doub
     tasks.push_back(t);
   }
   if (!run_grams(dg, tasks)) return false;
-  dg_chol_kernel<<<nb, 256, (size_t)J * J * sizeof(double), dg->st>>>(mass, mass_stride, linv, J, bad);
+  if (!keep_bytes(dg, &dg->d_shift, &dg->shift_cap, sizeof(int) * (size_t)nb * J)) return false;
+  int* shift = static_cast<int*>(dg->d_shift);
+  dg_chol_kernel<<<nb, 256, (size_t)J * J * sizeof(double), dg->st>>>(mass, mass_stride, linv, J, bad, shift);
   ++dg->launches;
   if (!cuda_ok(dg, cudaGetLastError(), "orthonormalisation")) return false;
   // phi = phi~ L^-T: L^-1 along the J axis of [1][J][n_LGL]
@@ -855,7 +693,7 @@ bool ortho_batch(dgdft_dg* dg, int nb, double* mass, long long mass_stride, doub
                     "pointer tables") &&
             cuda_ok(dg, cudaMemcpyAsync(d_out, cout.data(), cout.size() * sizeof(void*), cudaMemcpyHostToDevice, dg->st),
                     "pointer tables") &&
-            launch_axis(dg, d_in, d_out, nb, linv, J, J, dg->nL, 1, (long long)J * J) &&
+            launch_axis(dg, d_in, d_out, nb, linv, J, J, dg->nL, 1, (long long)J * J, shift) &&
             cuda_ok(dg, cudaStreamSynchronize(dg->st), "orthonormalisation");
   cudaFree(d_in);
   cudaFree(d_out);
@@ -881,7 +719,7 @@ bool ensure_batch(dgdft_dg* dg, int nb) {
 
 size_t batch_bytes(const dgdft_dg* dg) {
   const size_t per = (size_t)dg->J * dg->nL;
-  const size_t nchunk = (dg->nL + GR_CH - 1) / GR_CH;
+  const size_t chunk = gram_tensor_chunk(dg->nL), nchunk = (dg->nL + chunk - 1) / chunk;
   return sizeof(double) * ((size_t)dg->J * dg->ngq + dg->t1_elem + dg->t2_elem + 4 * per +
                            5 * nchunk * dg->J * dg->J);
 }
@@ -934,12 +772,12 @@ dgdft_status dgdft_dg_create(const dgdft_dg_config* cfg, dgdft_dg** out) {
   dg->nf[2] = dg->nl[0] * dg->nl[1];
   dg->t1_elem = (size_t)c.J * dg->nq[2] * dg->nq[1] * dg->nl[0];
   dg->t2_elem = (size_t)c.J * dg->nq[2] * dg->nl[1] * dg->nl[0];
-  // shared memory of every axis pass
-  size_t smax = axis_smem(c.J, c.J);
-  for (int d = 0; d < 3; ++d) smax = std::max({smax, axis_smem(dg->nq[d], dg->nl[d]), axis_smem(dg->nl[d], dg->nl[d])});
+  size_t smax = axis_size(c.J, c.J);
+  for (int d = 0; d < 3; ++d) smax = std::max({smax, axis_size(dg->nq[d], dg->nl[d]), axis_size(dg->nl[d], dg->nl[d])});
   if (smax > 220 * 1024) return dg->fail(DGDFT_EINVAL, "grids too large for the interpolation kernel");
-  if (!set_axis_smem<true>((int)smax) || !set_axis_smem<false>((int)smax) ||
-      cudaFuncSetAttribute(dg_chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (!dmalloc(&dg->d_terr, 1) || cudaMemset(dg->d_terr, 0, sizeof(int)) != cudaSuccess)
+    return dg->fail(DGDFT_ENOMEM, "status word");
+  if (cudaFuncSetAttribute(dg_chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(c.J * c.J * sizeof(double))) != cudaSuccess)
     return dg->fail(DGDFT_ECUDA, "kernel attributes");
   // tables
@@ -977,7 +815,9 @@ dgdft_status dgdft_dg_create(const dgdft_dg_config* cfg, dgdft_dg** out) {
   for (int d = 0; d < 3; ++d)
     if (!upload(dg, &dg->d_I[d], hI[d]) || !upload(dg, &dg->d_D[d], hD[d]) || !upload(dg, &dg->d_wf[d], hf[d]))
       return dg->fail(DGDFT_ENOMEM, "tables");
-  if (!upload(dg, &dg->d_w, hw)) return dg->fail(DGDFT_ENOMEM, "tables");
+  std::vector<double> hs(hw);
+  for (double& x : hs) x = std::sqrt(x);
+  if (!upload(dg, &dg->d_w, hw) || !upload(dg, &dg->d_sw, hs)) return dg->fail(DGDFT_ENOMEM, "tables");
   // neighbourhoods and block rows
   dg->nb.resize(dg->nel);
   dg->row_first.resize(dg->nel + 1, 0);
@@ -1357,6 +1197,7 @@ dgdft_status dgdft_dg_assemble(dgdft_dg* dg, const double* const* z, int on_devi
   for (void* p : {(void*)d_terms, (void*)d_kbt, (void*)d_term_ptr, (void*)d_kbp}) cudaFree(p);
   cleanup();
   if (!ok) return DGDFT_ECUDA;
+  if (!tensor_waits_ok(dg)) return DGDFT_ETIMEOUT;
   std::vector<int> bad(nel);
   if (cudaMemcpy(bad.data(), dg->d_bad, sizeof(int) * nel, cudaMemcpyDeviceToHost) != cudaSuccess)
     return dg->fail(DGDFT_ECUDA, "status copy");
@@ -1410,6 +1251,7 @@ dgdft_status dgdft_dg_lgl_basis(dgdft_dg* dg, int elem, const double* z, int z_o
   cudaFree(d_linv);
   cudaFree(d_bad);
   if (!ok) return DGDFT_ECUDA;
+  if (!tensor_waits_ok(dg)) return DGDFT_ETIMEOUT;
   if (bad) return dg->fail(DGDFT_ENOTCONV, "mass matrix is not positive definite");
   return DGDFT_OK;
 }
@@ -1549,7 +1391,8 @@ dgdft_status dgdft_dg_density(dgdft_dg* dg, const double* const* z, int z_on_dev
   dg->density_ms[0] = t_ms[0];
   dg->density_ms[1] = t_ms[1];
   release();
-  return ok ? DGDFT_OK : DGDFT_ECUDA;
+  if (!ok) return DGDFT_ECUDA;
+  return tensor_waits_ok(dg) ? DGDFT_OK : DGDFT_ETIMEOUT;
 }
 
 dgdft_status dgdft_dg_density_info(dgdft_dg* dg, int* sweeps) {
@@ -1576,9 +1419,10 @@ void dgdft_dg_destroy(dgdft_dg* dg) {
     cudaFree(dg->d_wf[d]);
     cudaFree(dg->d_g[d]);
   }
-  for (void* p : {(void*)dg->d_w, (void*)dg->d_v, (void*)dg->d_pool, (void*)dg->d_traces, (void*)dg->d_linv,
+  for (void* p : {(void*)dg->d_w, (void*)dg->d_sw, (void*)dg->d_v, (void*)dg->d_pool, (void*)dg->d_traces, (void*)dg->d_linv,
                   (void*)dg->d_H, (void*)dg->d_bad, (void*)dg->d_z, (void*)dg->d_t1,
-                  (void*)dg->d_t2, (void*)dg->d_phi, (void*)dg->d_part, (void*)dg->d_eig})
+                  (void*)dg->d_t2, (void*)dg->d_phi, (void*)dg->d_part, (void*)dg->d_eig, dg->d_img, dg->d_shift,
+                  dg->d_tasks, (void*)dg->d_terr})
     cudaFree(p);
   delete dg;
 }
