@@ -7,8 +7,9 @@
 // (split-K) and the partial products are summed on the device in a fixed
 // order, so results do not depend on scheduling.
 //
-// These are the SIMT kernels (FP64 for the plain solver, FP32 accumulation
-// within a chunk for the mixed form); partial sums are always FP64.
+// These are the SIMT kernels of the FP32 stage (the FP64 stage's products and
+// updates run on the tensor cores, fp64_tensor.cu; tsmm_kernel<double> takes
+// updates of more than 1,024 input columns); partial sums are always FP64.
 #include "internal.h"
 
 namespace dgdft {
@@ -220,253 +221,6 @@ __global__ void __launch_bounds__(144) gram48_kernel(const ElemDev<float>* __res
     for (int j = 0; j < 4; ++j) out[(ty * 4 + i) * TILE + tx * 4 + j] = (double)chi[i][j] + (double)clo[i][j];
 }
 
-// FP64 Gram products for blocks of at most 48 columns (the FP64 stage at
-// m <= 48): the layout of gram48_kernel with 16-row stages of doubles, each
-// thread reading 2 rows of a column as one 16-byte double2 (chunks of a
-// column swizzled by column group as there).  FP64 accumulation; the FP64
-// pipe bounds it, and 48-wide tiles avoid the 64-wide tiles' idle lanes.
-// Narrow blocks take only the ceil(m/4)^2 threads of one tile per row group:
-// the CTA's threads form up to eight groups that share a stage's rows and add
-// up at the end, so that no FP64 instruction works on columns past m (m = 16,
-// 4,096 rows: 1,420 us per launch with all threads on the 48-wide tile and two
-// chunks, 32 us with eight groups and launch_gram's shorter chunks).
-// grid: (npairs, nchunk, nel); block 144.
-constexpr int GKD = 16;  // rows per stage (doubles)
-
-__device__ __forceinline__ int g48d_off(int c, int r) {
-  return c * GKD + ((((r >> 1) ^ ((c >> 2) & 7)) << 1) | (r & 1));
-}
-
-__global__ void __launch_bounds__(144) gram48d_kernel(const ElemDev<double>* __restrict__ elems,
-                                                       GramJob<double> job, double* __restrict__ partial,
-                                                       size_t pstride, int kchunk) {
-  __shared__ __align__(16) double As[2][G48 * GKD];
-  __shared__ __align__(16) double Bs[2][G48 * GKD];
-  const ElemDev<double>& e = elems[blockIdx.z];
-  if (!e.state[ST_ACTIVE]) return;
-  const int pair = blockIdx.x;
-  if (job.needs_p[pair] && !e.state[ST_HAS_P]) return;
-  const int ca = job.ncols_a > 0 ? job.ncols_a : e.m;
-  const int cb = job.ncols_b > 0 ? job.ncols_b : e.m;
-  const int rows = job.rows > 0 ? job.rows : e.ng;
-  const double* A = resolve(e, job.a[pair]);
-  const double* B = resolve(e, job.b[pair]);
-  const int lda = ld_of(e, job.a[pair], job.ld_in, rows);
-  const int ldb = ld_of(e, job.b[pair], job.ld_in, rows);
-  // tile of td x td threads (4 x 4 outputs each), ngrp groups of them
-  const int td = (max(ca, cb) + 3) / 4;
-  const int ngrp = min(8, 144 / (td * td));
-  const int grp = threadIdx.x / (td * td), tt = threadIdx.x - grp * td * td;
-  const int tx = tt % td, ty = tt / td;
-  const int k_beg = blockIdx.y * kchunk;
-  const int k_end = min(rows, k_beg + kchunk);
-  const bool vec = ((lda | ldb | k_beg) & 1) == 0 && ((((uintptr_t)A) | ((uintptr_t)B)) & 15) == 0;
-  auto load_stage = [&](int buf, int k0) {
-    for (int t = threadIdx.x; t < 2 * G48 * (GKD / 2); t += blockDim.x) {
-      const int op = t / (G48 * (GKD / 2));
-      const int rem = t - op * (G48 * (GKD / 2));
-      const int c = rem / (GKD / 2), q = rem - c * (GKD / 2);
-      const double* src = op ? B : A;
-      const int ld = op ? ldb : lda;
-      const int cc = op ? cb : ca;
-      double* dst = (op ? Bs[buf] : As[buf]) + g48d_off(c, 2 * q);
-      const int k = k0 + 2 * q;
-      const int nv = (c < cc) ? max(0, min(2, k_end - k)) : 0;
-      const double* g = nv ? src + (size_t)c * ld + k : src;
-      if (vec) {
-        cp_async16(dst, g, 8 * nv);
-      } else {
-        // 8-byte pieces: two 4-byte copies each
-        const float* gf = reinterpret_cast<const float*>(g);
-        const float* sf = reinterpret_cast<const float*>(src);
-        float* df = reinterpret_cast<float*>(dst);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) cp_async4(df + u, u < 2 * nv ? gf + u : sf, u < 2 * nv ? 4 : 0);
-      }
-    }
-    cp_async_commit();
-  };
-  double acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-  const int nst = (k_end > k_beg) ? (k_end - k_beg + GKD - 1) / GKD : 0;
-  if (nst > 0) load_stage(0, k_beg);
-  for (int st = 0; st < nst; ++st) {
-    if (st + 1 < nst) {
-      load_stage((st + 1) & 1, k_beg + (st + 1) * GKD);
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
-    __syncthreads();
-    const double* as = As[st & 1];
-    const double* bs = Bs[st & 1];
-    if (grp < ngrp)
-#pragma unroll 2
-    for (int r = 2 * grp; r < GKD; r += 2 * ngrp) {
-      double2 a2[4], b2[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a2[i] = *reinterpret_cast<const double2*>(as + g48d_off(ty * 4 + i, r));
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b2[j] = *reinterpret_cast<const double2*>(bs + g48d_off(tx * 4 + j, r));
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a2[i].y, b2[j].y, fma(a2[i].x, b2[j].x, acc[i][j]));
-    }
-    __syncthreads();
-  }
-  if (ngrp > 1) {
-    // the groups' sums, added in group order (a group holds at most 36 threads)
-    double* sums = &As[0][0];
-    for (int g = 1; g < ngrp; ++g) {
-      if (grp == g)
-#pragma unroll
-        for (int q = 0; q < 16; ++q) sums[q * (td * td) + tt] = acc[q >> 2][q & 3];
-      __syncthreads();
-      if (grp == 0)
-#pragma unroll
-        for (int q = 0; q < 16; ++q) acc[q >> 2][q & 3] += sums[q * (td * td) + tt];
-      __syncthreads();
-    }
-    if (grp > 0) return;
-  } else if (grp > 0) {
-    return;
-  }
-  double* out = partial + blockIdx.z * pstride + ((size_t)blockIdx.y * gridDim.x + pair) * (TILE * TILE);
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) out[(ty * 4 + i) * TILE + tx * 4 + j] = acc[i][j];
-}
-
-// FP64 Gram products in double-float arithmetic (the FP64 stage at m <= 48).
-// GB300 runs FP64 at 1/64 of the FP32 rate, and gram48d_kernel is bound by
-// it.  Here each staged FP64 value x is split once into FP32 parts
-// x = xh + xl (|xl| <= 2^-24 |xh|, the pair carries ~2^-48 of x); a product
-// is formed as xh*yh exactly (its rounding error recovered by an FMA) plus
-// the cross terms xh*yl + xl*yh, and accumulated into a (hi, lo) FP32 pair
-// by a two-sum per product: ~2^-44 relative, at FP32-pipe rates.  The FP64
-// stage only needs its pencil far more accurately than the FP32 stage's,
-// not to FP64 rounding.  Layout and staging as gram48d_kernel (FP64 blocks
-// staged by cp.async), then a conversion pass writes the parts row-major
-// ([row][column], 48 floats a row) so a thread reads its four columns as
-// one float4.  grid: (npairs, nchunk, nel); block 144.
-__global__ void __launch_bounds__(144) gram48df_kernel(const ElemDev<double>* __restrict__ elems,
-                                                        GramJob<double> job, double* __restrict__ partial,
-                                                        size_t pstride, int kchunk) {
-  __shared__ __align__(16) double As[2][G48 * GKD];
-  __shared__ __align__(16) double Bs[2][G48 * GKD];
-  __shared__ __align__(16) float Ah[GKD][G48], Al[GKD][G48], Bh[GKD][G48], Bl[GKD][G48];
-  const ElemDev<double>& e = elems[blockIdx.z];
-  if (!e.state[ST_ACTIVE]) return;
-  const int pair = blockIdx.x;
-  if (job.needs_p[pair] && !e.state[ST_HAS_P]) return;
-  const int ca = job.ncols_a > 0 ? job.ncols_a : e.m;
-  const int cb = job.ncols_b > 0 ? job.ncols_b : e.m;
-  const int rows = job.rows > 0 ? job.rows : e.ng;
-  const double* A = resolve(e, job.a[pair]);
-  const double* B = resolve(e, job.b[pair]);
-  const int lda = ld_of(e, job.a[pair], job.ld_in, rows);
-  const int ldb = ld_of(e, job.b[pair], job.ld_in, rows);
-  const int tx = threadIdx.x % 12, ty = threadIdx.x / 12;
-  const int k_beg = blockIdx.y * kchunk;
-  const int k_end = min(rows, k_beg + kchunk);
-  const bool vec = ((lda | ldb | k_beg) & 1) == 0 && ((((uintptr_t)A) | ((uintptr_t)B)) & 15) == 0;
-  auto load_stage = [&](int buf, int k0) {
-    for (int t = threadIdx.x; t < 2 * G48 * (GKD / 2); t += blockDim.x) {
-      const int op = t / (G48 * (GKD / 2));
-      const int rem = t - op * (G48 * (GKD / 2));
-      const int c = rem / (GKD / 2), q = rem - c * (GKD / 2);
-      const double* src = op ? B : A;
-      const int ld = op ? ldb : lda;
-      const int cc = op ? cb : ca;
-      double* dst = (op ? Bs[buf] : As[buf]) + g48d_off(c, 2 * q);
-      const int k = k0 + 2 * q;
-      const int nv = (c < cc) ? max(0, min(2, k_end - k)) : 0;
-      const double* g = nv ? src + (size_t)c * ld + k : src;
-      if (vec) {
-        cp_async16(dst, g, 8 * nv);
-      } else {
-        const float* gf = reinterpret_cast<const float*>(g);
-        const float* sf = reinterpret_cast<const float*>(src);
-        float* df = reinterpret_cast<float*>(dst);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) cp_async4(df + u, u < 2 * nv ? gf + u : sf, u < 2 * nv ? 4 : 0);
-      }
-    }
-    cp_async_commit();
-  };
-  float sh[4][4], sl[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) sh[i][j] = sl[i][j] = 0.f;
-  const int nst = (k_end > k_beg) ? (k_end - k_beg + GKD - 1) / GKD : 0;
-  if (nst > 0) load_stage(0, k_beg);
-  for (int st = 0; st < nst; ++st) {
-    if (st + 1 < nst) {
-      load_stage((st + 1) & 1, k_beg + (st + 1) * GKD);
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
-    __syncthreads();
-    // split the stage into FP32 parts, transposed to [row][column]
-    for (int t = threadIdx.x; t < 2 * G48 * GKD; t += blockDim.x) {
-      const int op = t / (G48 * GKD);
-      const int rem = t - op * (G48 * GKD);
-      const int c = rem / GKD, r = rem - c * GKD;
-      const double x = (op ? Bs[st & 1] : As[st & 1])[g48d_off(c, r)];
-      const float h = __double2float_rn(x);
-      const float l = __double2float_rn(x - (double)h);
-      (op ? Bh : Ah)[r][c] = h;
-      (op ? Bl : Al)[r][c] = l;
-    }
-    __syncthreads();
-#pragma unroll 2
-    for (int r = 0; r < GKD; ++r) {
-      const float4 ah = *reinterpret_cast<const float4*>(&Ah[r][ty * 4]);
-      const float4 al = *reinterpret_cast<const float4*>(&Al[r][ty * 4]);
-      const float4 bh = *reinterpret_cast<const float4*>(&Bh[r][tx * 4]);
-      const float4 bl = *reinterpret_cast<const float4*>(&Bl[r][tx * 4]);
-      const float a_h[4] = {ah.x, ah.y, ah.z, ah.w}, a_l[4] = {al.x, al.y, al.z, al.w};
-      const float b_h[4] = {bh.x, bh.y, bh.z, bh.w}, b_l[4] = {bl.x, bl.y, bl.z, bl.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float p = __fmul_rn(a_h[i], b_h[j]);              // never contracted into the sum
-          const float pe = fmaf(a_h[i], b_h[j], -p);           // exact: p + pe = a_h b_h
-          const float cr = fmaf(a_h[i], b_l[j], a_l[i] * b_h[j]);
-          const float s = sh[i][j] + p;                          // two-sum of sh and p
-          const float bp = s - sh[i][j];
-          const float err = (sh[i][j] - (s - bp)) + (p - bp);
-          sh[i][j] = s;
-          sl[i][j] += err + (pe + cr);
-        }
-    }
-    // renormalise the pairs: the low part stays within a few units of the
-    // high part's last place, so its own rounding stays at ~2^-48 of it
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float t = sh[i][j] + sl[i][j];
-        sl[i][j] -= t - sh[i][j];
-        sh[i][j] = t;
-      }
-    __syncthreads();
-  }
-  double* out = partial + blockIdx.z * pstride + ((size_t)blockIdx.y * gridDim.x + pair) * (TILE * TILE);
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) out[(ty * 4 + i) * TILE + tx * 4 + j] = (double)sh[i][j] + (double)sl[i][j];
-}
-
 template <class real>
 __global__ void gram_reduce_kernel(const ElemDev<real>* __restrict__ elems, GramJob<real> job,
                                    const double* __restrict__ partial, size_t pstride, int nchunk,
@@ -571,110 +325,6 @@ __global__ void __launch_bounds__(256) tsmm_kernel(const ElemDev<real>* __restri
       real* o = O + (size_t)col * ldo + row;
       real v = (real)job.alpha * acc[i][j];
       if (job.beta != 0.0) v += (real)job.beta * *o;
-      *o = v;
-    }
-  }
-}
-
-// FP64 block update in double-float arithmetic (the mixed form's FP64 stage):
-// the tiling of tsmm_kernel, with every staged block and coefficient value
-// split into FP32 parts (x = xh + xl) and each output accumulated as a
-// (hi, lo) FP32 pair: exact leading products by FMA, cross terms, a two-sum
-// per product (~2^-44 relative, at FP32-pipe rates).  alpha and beta are
-// applied in FP64 to the pair's sum.
-__global__ void __launch_bounds__(256) tsmm_df_kernel(const ElemDev<double>* __restrict__ elems,
-                                                       TsmmJob<double> job) {
-  __shared__ float Sh[KU][TILE + 4], Sl[KU][TILE + 4];
-  __shared__ float Yh[KU][TILE + 4], Yl[KU][TILE + 4];
-  const ElemDev<double>& e = elems[blockIdx.z];
-  if (!e.state[ST_ACTIVE]) return;
-  const int nc = job.ncols > 0 ? job.ncols : e.m;
-  const int rows = job.rows > 0 ? job.rows : e.ng;
-  const int r0 = blockIdx.x * TILE, c0 = blockIdx.y * TILE;
-  if (r0 >= rows || c0 >= nc) return;
-  const double* Y;
-  int ldy;
-  switch (job.y_id) {
-    case Y_RR: Y = e.Y; ldy = job.ldy > 0 ? job.ldy : 3 * e.m; break;
-    case Y_GXW: Y = e.gxw; ldy = job.ldy > 0 ? job.ldy : e.m; break;
-    default: Y = job.y_ptr; ldy = job.ldy; break;
-  }
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  float ah[4][4], al[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) ah[i][j] = al[i][j] = 0.f;
-  const int ycol0 = job.ycol * nc + c0;
-  for (int in = 0; in < job.nin; ++in) {
-    if (job.needs_p[in] && !e.state[ST_HAS_P]) continue;
-    const double* S = resolve(e, job.in[in]);
-    const int lds = ld_of(e, job.in[in], job.ld_in, rows);
-    const int yrow0 = job.yrow[in] * nc;
-    for (int k0 = 0; k0 < nc; k0 += KU) {
-      for (int i = threadIdx.x; i < KU * TILE; i += blockDim.x) {
-        const int kk = i / TILE, r = i - kk * TILE;
-        const bool kin = k0 + kk < nc;
-        const double sv = (kin && r0 + r < rows) ? S[(size_t)(k0 + kk) * lds + r0 + r] : 0.0;
-        const double yv = (kin && c0 + r < nc) ? Y[(yrow0 + k0 + kk) + (size_t)(ycol0 + r) * ldy] : 0.0;
-        const float svh = __double2float_rn(sv), yvh = __double2float_rn(yv);
-        Sh[kk][r] = svh;
-        Sl[kk][r] = __double2float_rn(sv - (double)svh);
-        Yh[kk][r] = yvh;
-        Yl[kk][r] = __double2float_rn(yv - (double)yvh);
-      }
-      __syncthreads();
-#pragma unroll
-      for (int kk = 0; kk < KU; ++kk) {
-        float sh[4], sl[4], yh[4], yl[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          sh[i] = Sh[kk][tx + 16 * i];
-          sl[i] = Sl[kk][tx + 16 * i];
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          yh[j] = Yh[kk][ty * 4 + j];
-          yl[j] = Yl[kk][ty * 4 + j];
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float p = __fmul_rn(sh[i], yh[j]);  // never contracted into the sum
-            const float pe = fmaf(sh[i], yh[j], -p);
-            const float cr = fmaf(sh[i], yl[j], sl[i] * yh[j]);
-            const float t = ah[i][j] + p;
-            const float bp = t - ah[i][j];
-            const float err = (ah[i][j] - (t - bp)) + (p - bp);
-            ah[i][j] = t;
-            al[i][j] += err + (pe + cr);
-          }
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float t = ah[i][j] + al[i][j];
-          al[i][j] -= t - ah[i][j];
-          ah[i][j] = t;
-        }
-      __syncthreads();
-    }
-  }
-  double* O = resolve(e, job.out);
-  const int ldo = ld_of(e, job.out, job.ld_in, rows);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int col = c0 + ty * 4 + j;
-    if (col >= nc) continue;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int row = r0 + tx + 16 * i;
-      if (row >= rows) continue;
-      double* o = O + (size_t)col * ldo + row;
-      double v = job.alpha * ((double)ah[i][j] + (double)al[i][j]);
-      if (job.beta != 0.0) v += job.beta * *o;
       *o = v;
     }
   }
@@ -1125,23 +775,18 @@ void launch_gram(const Batch<real>& b, const GramJob<real>& job, double* partial
   int kchunk = 2048;
   while (kchunk > 128 && (size_t)((rows + kchunk - 1) / kchunk) * ny * s.nel < 304) kchunk /= 2;
   int nchunk = (rows + kchunk - 1) / kchunk;
-  while ((size_t)nchunk * ny * TILE * TILE * s.nel > partial_cap && kchunk < (1 << 30)) {
+  size_t exps = 0;
+  if constexpr (std::is_same<real, double>::value) exps = (gram_dig_ints(job, ca, cb, s.nel) + 1) / 2;
+  while ((size_t)nchunk * ny * TILE * TILE * s.nel + exps > partial_cap && kchunk < (1 << 30)) {
     kchunk *= 2;
     nchunk = (rows + kchunk - 1) / kchunk;
   }
   const size_t pstride = (size_t)nchunk * ny * TILE * TILE;
-  if (std::is_same<real, float>::value && ca <= G48 && cb <= G48) {
-    gram48_kernel<<<dim3(ny, nchunk, s.nel), 144, 0, st>>>(
-        reinterpret_cast<const ElemDev<float>*>(b.d_elems), *reinterpret_cast<const GramJob<float>*>(&job), partial,
-        pstride, kchunk);
-  } else if (std::is_same<real, double>::value && ca <= G48 && cb <= G48 && s.dfloat) {
-    gram48df_kernel<<<dim3(ny, nchunk, s.nel), 144, 0, st>>>(
-        reinterpret_cast<const ElemDev<double>*>(b.d_elems), *reinterpret_cast<const GramJob<double>*>(&job),
-        partial, pstride, kchunk);
-  } else if (std::is_same<real, double>::value && ca <= G48 && cb <= G48) {
-    gram48d_kernel<<<dim3(ny, nchunk, s.nel), 144, 0, st>>>(
-        reinterpret_cast<const ElemDev<double>*>(b.d_elems), *reinterpret_cast<const GramJob<double>*>(&job),
-        partial, pstride, kchunk);
+  if constexpr (std::is_same<real, double>::value) {
+    // the exponents of the columns lie behind the partials
+    launch_gram_dig(b, job, partial, pstride, kchunk, nchunk, ca, cb, reinterpret_cast<int*>(partial + pstride * s.nel), st);
+  } else if (ca <= G48 && cb <= G48) {
+    gram48_kernel<<<dim3(ny, nchunk, s.nel), 144, 0, st>>>(b.d_elems, job, partial, pstride, kchunk);
   } else {
     gram_kernel<real><<<dim3(nchunk, ny, s.nel), 256, 0, st>>>(b.d_elems, job, partial, pstride, kchunk,
                                                                tiles_a, tiles_b);
@@ -1169,11 +814,7 @@ void launch_tsmm(const Batch<real>& b, const TsmmJob<real>& job, cudaStream_t st
   }
   const int rows = job.rows > 0 ? job.rows : s.max_ng;
   if constexpr (std::is_same<real, double>::value) {
-    if (s.dfloat) {
-      tsmm_df_kernel<<<dim3((rows + TILE - 1) / TILE, (nc + TILE - 1) / TILE, s.nel), 256, 0, st>>>(b.d_elems,
-                                                                                                  job);
-      return;
-    }
+    if (launch_update_dig(b, job, st)) return;
   }
   tsmm_kernel<real><<<dim3((rows + TILE - 1) / TILE, (nc + TILE - 1) / TILE, s.nel), 256, 0, st>>>(
       b.d_elems, job);
@@ -1217,7 +858,10 @@ void launch_iter_finish(const Batch<real>& b, int set_p, cudaStream_t st) {
   iter_finish_kernel<real><<<(b.s.nel + 127) / 128, 128, 0, st>>>(b.d_elems, b.s.nel, set_p);
 }
 
-void init_blas_kernels() { opt_in_dynamic_smem((const void*)tsmm_rows_kernel); }
+void init_blas_kernels() {
+  opt_in_dynamic_smem((const void*)tsmm_rows_kernel);
+  init_fp64_tensor_kernels();
+}
 
 #define DGDFT_INST(real)                                                                             \
   template void launch_gram<real>(const Batch<real>&, const GramJob<real>&, double*, size_t,         \

@@ -16,7 +16,7 @@
 #include <algorithm>
 
 #include "dg_tensor.h"
-#include "digits.cuh"
+#include "dig_gram.cuh"
 #include "internal.h"
 
 namespace dgdft {
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(DIG_THREADS, 1) axis_tensor_kernel(AxisShape j
           if (j >= nout || gr >= lines) continue;
           if (NKS) dst[(long long)j * S] = dig_value(t[u], er, fs[j]);
           else
-            dst[(long long)j * S] = dig_value_sum(hs[(4 * q + u) % (NKS ? 1 : NB / 4)],
+            dst[(long long)j * S] = dig_value_sum<DIG>(hs[(4 * q + u) % (NKS ? 1 : NB / 4)],
                                                   ls[(4 * q + u) % (NKS ? 1 : NB / 4)], er, fs[j]);
         }
       }
@@ -302,14 +302,9 @@ __global__ void __launch_bounds__(256) gram_exp_kernel(const TGramTask* __restri
   }
 }
 
-// X^T diag(w v) Y, item (task, row chunk, chunk of NB columns of Y): rows of the
-// product are the columns of X (`arows`, up to 128, in shared memory), K the
-// points.  sym: (w X)^T (w X), one operand for both sides.  A thread splits
-// groups of eight points g, g + 8, .. of one column (neighbouring threads read
-// neighbouring points): group t, t + 512, ... of (columns x 8) per stage.  DB:
-// two buffers of operands, so that a stage's products run while the next one
-// is split; otherwise (more than 80 columns) one.  Exact integer sums over the
-// whole chunk; partials as dg_gram_reduce_kernel reads them.
+// X^T diag(w v) Y, item (task, row chunk, chunk of NB columns of Y); sym: (w X)^T
+// (w X).  DB: two operand buffers, where at most 112 columns have to fit.
+// Partials as dg_gram_reduce_kernel reads them.
 template <int NB, int RT, bool DB>
 __global__ void __launch_bounds__(DIG_THREADS, 1) gram_tensor_kernel(const TGramTask* __restrict__ tasks,
                                                                      const int* __restrict__ items, int nitems, int arows,
@@ -321,137 +316,36 @@ __global__ void __launch_bounds__(DIG_THREADS, 1) gram_tensor_kernel(const TGram
   __shared__ int abort_s;
   __shared__ DigWeight ws[2][DIG_K];  // weights of this stage and the next
   unsigned char* base = reinterpret_cast<unsigned char*>(((uintptr_t)dig_raw + 1023) & ~(uintptr_t)1023);
-  const int astep = arows * 128, boff = DIG * astep, buf = boff + DIG * NB * 128;
-  const uint32_t abase = smem_u32(base);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (tid == 0) abort_s = 0;
+  if (threadIdx.x == 0) abort_s = 0;
   DigCta cta;
   dig_open(cta, bar, &slot);
   for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
     const TGramTask T = tasks[items[3 * it]];
     const int chunk = items[3 * it + 1], j0 = items[3 * it + 2] * NB;
-    const int nB = min(NB, T.J2 - j0), rows = T.J1 + (T.sym ? 0 : nB);
-    const int p0 = chunk * T.chunk, p1 = min(T.n, p0 + T.chunk);
-    double v[RT][8];
-    auto load = [&](int p) {
-#pragma unroll
-      for (int k = 0; k < RT; ++k) {
-        const int q = tid + k * DIG_THREADS, r = q >> 3, pt = p + (q & 7);
-        const bool left = r < T.J1;
-        const double* col = left ? T.X + (size_t)r * T.ldx : T.Y + (size_t)(j0 + r - T.J1) * T.ldy;
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[k][u] = (r < rows && pt + 8 * u < p1) ? col[pt + 8 * u] : 0.0;
-      }
-    };
-    // weight of point p + tid, tid < 64
-    auto weight = [&](int p) {
-      const int pt = p + tid;
-      double w = (tid < DIG_K && pt < p1) ? T.w[pt] : 0.0;
-      if (T.v && tid < DIG_K && pt < p1) w *= T.v[pt];
-      return w;
-    };
-    int ek[RT];  // exponents of this thread's columns
-#pragma unroll
-    for (int k = 0; k < RT; ++k) {
-      const int r = (tid + k * DIG_THREADS) >> 3;
-      ek[k] = r < rows ? exps[T.exp0 + (r < T.J1 ? r : j0 + r)] : 64;
-    }
-    long long hs[NB / 4], ls[NB / 4];
-#pragma unroll
-    for (int q = 0; q < NB / 4; ++q) hs[q] = ls[q] = 0;
-    if (tid < DIG_K) ws[0][tid] = dig_weight(weight(p0));
-    __syncthreads();
-    const int nst = (p1 - p0 + DIG_K - 1) / DIG_K;
-    // the products of stage st are done; the sums of a window are read (by the
-    // warps whose rows and columns are in use)
-    auto finish = [&](int st) {
-      dig_wait(cta, &abort_s);
-      if ((st % DIG_WINDOW) != DIG_WINDOW - 1 && st != nst - 1) return;
-      const uint32_t ta = cta.tmem + ((uint32_t)((warp & 3) * 32) << 16);
-      if ((warp & 3) * 32 < T.J1) {
-#pragma unroll
-        for (int q = 0; q < NB / 16; ++q) {
-          const int c0 = (warp >> 2) * 4 + 16 * q;
-          if (c0 >= nB) continue;
-          long long hi[4], lo[4];
-          dig_drain4<NB>(ta + c0, hi, lo);
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            hs[4 * q + u] += hi[u];
-            ls[4 * q + u] += lo[u];
-          }
-        }
-      }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    };
-    load(p0);
-    for (int st = 0; st < nst; ++st) {
-      const int p = p0 + st * DIG_K, off = DB ? (st & 1) * buf : 0;
-      if (!DB && st > 0) finish(st - 1);
-#pragma unroll
-      for (int k = 0; k < RT; ++k) {
-        const int q = tid + k * DIG_THREADS, r = q >> 3, g = q & 7;
-        if (r >= rows) continue;
-        const bool left = r < T.J1;
-        uint4 d[DIG];
-        if (left) dig_split8w(v[k], &ws[st & 1][g], 8, ek[k], d);
-        else dig_split8(v[k], ek[k], d);
-        unsigned char* dst = base + off + (left ? dig_off(r, g) : boff + dig_off(r - T.J1, g));
-        const int step = left ? astep : NB * 128;
-#pragma unroll
-        for (int i = 0; i < DIG; ++i) *reinterpret_cast<uint4*>(dst + i * step) = d[i];
-      }
-      const double wn = weight(p + DIG_K);
-      if (st + 1 < nst) load(p + DIG_K);
-      if (DB && st > 0) finish(st - 1);
-      if (tid < DIG_K) ws[(st + 1) & 1][tid] = dig_weight(wn);
-      dig_publish();
-      dig_launch<NB>(cta, abase + off, astep, abase + off + (T.sym ? 0 : boff), 4, (st % DIG_WINDOW) == 0);
-    }
-    finish(nst - 1);
-    const int r = (warp & 3) * 32 + lane;
-    if (r < T.J1) {
-      double* out = partial + T.part + (size_t)chunk * T.J1 * T.J2 + (size_t)r * T.J2;
-      const int e = exps[T.exp0 + r];
-#pragma unroll
-      for (int q = 0; q < NB / 16; ++q)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int c = (warp >> 2) * 4 + 16 * q + u;
-          if (c >= nB) continue;
-          const int f = exps[T.exp0 + (T.sym ? 0 : T.J1) + j0 + c];
-          out[j0 + c] = dig_value_sum(hs[4 * q + u], ls[4 * q + u], e, f);
-        }
-    }
+    DigGramOp op;
+    op.X = T.X;
+    op.Y = T.Y + (size_t)j0 * T.ldy;
+    op.ldx = T.ldx;
+    op.ldy = T.ldy;
+    op.w = T.w;
+    op.v = T.v;
+    op.ex = exps + T.exp0;
+    op.ey = op.ex + T.J1 + j0;
+    op.J1 = T.J1;
+    op.nB = min(NB, T.J2 - j0);
+    op.p0 = chunk * T.chunk;
+    op.p1 = min(T.n, op.p0 + T.chunk);
+    op.sym = T.sym != 0;
+    dig_gram_chunk<NB, RT, DB, true, DIG>(cta, op, base, arows, ws, &abort_s,
+                                     partial + T.part + (size_t)chunk * T.J1 * T.J2 + j0, T.J2);
     __syncthreads();
     if (abort_s) break;
   }
-  if (abort_s && tid == 0) atomicExch(err, 1);
+  if (abort_s && threadIdx.x == 0) atomicExch(err, 1);
   dig_close(cta, bar + 1, abort_s != 0);
 }
 
-int sm_count() {
-  int dev = 0, n = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-  return n;
-}
-
-// columns of B per chunk: a multiple of 16, at most 64 (seven blocks of
-// accumulators in tensor memory), the chunks as even as can be
-int chunk_cols(int n) {
-  const int c = (n + 63) / 64;
-  return ((n + c - 1) / c + 15) / 16 * 16;
-}
-
-// dynamic shared memory a CTA can have beside 3 KB of static
-constexpr size_t DIG_SMEM_MAX = 232448 - 3200;
-
 size_t dig_smem(int nb, int images) { return (size_t)DIG * DIG_A_BYTES + (size_t)images * DIG * nb * 128 + 1024; }
-
-template <class K> void dig_opt_in(K k, size_t smem) {
-  cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
 
 template <int NB> void launch_axis_nb(const AxisShape& s, int grid, size_t smem, cudaStream_t st) {
   if (s.nks > 2) {

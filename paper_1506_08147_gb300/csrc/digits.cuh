@@ -105,6 +105,52 @@ __device__ __forceinline__ void dig_split8(const double (&x)[8], int e, uint4 (&
   dig_bytes8(lo, hi, sg, q);
 }
 
+// Eight digits where a sum has few terms, so that seven's dropped orders (rms
+// 2^-53 of the largest product a term) would show: X = x 2^(1084 - e), |X| < 2^62,
+// the 36 products with i + j <= 7; the result is exact to 2^-60 of the product of
+// the largest entries, and entries above 2^-9 of them keep all their bits.
+constexpr int DIG8 = 8;
+
+// Eight digits of eight entries, entry u standing for x[u] 2^s[u] (e at least
+// their exponents).
+__device__ __forceinline__ void dig8_split8s(const double (&x)[8], const int (&s)[8], int e, uint4 (&q)[DIG8]) {
+  uint32_t r[DIG8][4];
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    uint32_t lo[2], hi[2], sg[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int u = 2 * p + c;
+      const uint32_t h = (uint32_t)__double2hiint(x[u]), l = (uint32_t)__double2loint(x[u]);
+      const int ex = (h >> 20) & 0x7ff;
+      const int sh = ex == 0 ? 63 : max(min(e - ex - s[u], 63), 0);
+      unsigned long long m = ((unsigned long long)((h & 0xfffffu) | 0x100000u) << 41) | ((unsigned long long)l << 9);
+      m = (m >> sh) + 0x8080808080808080ull;
+      sg[c] = h;
+      lo[c] = (uint32_t)m;
+      hi[c] = (uint32_t)(m >> 32);
+    }
+    const uint32_t o = (__byte_perm(sg[0], sg[1], 0x7632) & 0x80008000u) | 0x3c003c00u;  // +-1
+    const __half2 one = *reinterpret_cast<const __half2*>(&o);
+    const __half2 off = __hmul2(one, __floats2half2_rn(-1152.0f, -1152.0f));
+    auto put = [&](int i, uint32_t w) {
+      const __half2 d = __hfma2(*reinterpret_cast<const __half2*>(&w), one, off);
+      r[i][p] = *reinterpret_cast<const uint32_t*>(&d);
+    };
+    auto word = [&](int i, uint32_t a, uint32_t b) {  // four digits of a 32-bit half
+      const uint32_t ma = __byte_perm(a, 0x64u, 0x4321), mb = __byte_perm(b, 0x64u, 0x4321);
+      put(i, __byte_perm(ma, mb, 0x7632));
+      put(i + 1, __byte_perm(ma, mb, 0x7531));
+      put(i + 2, __byte_perm(ma, mb, 0x7430));
+      put(i + 3, (__byte_perm(a, b, 0x4400) & 0x00ff00ffu) | 0x64006400u);
+    };
+    word(0, hi[0], hi[1]);
+    word(4, lo[0], lo[1]);
+  }
+#pragma unroll
+  for (int i = 0; i < DIG8; ++i) q[i] = make_uint4(r[i][0], r[i][1], r[i][2], r[i][3]);
+}
+
 // A weight: its mantissa left-aligned, the leading bit (always 1) replaced by
 // the sign, and its exponent; a zero's (or a subnormal's) is far below any entry's
 struct DigWeight {
@@ -161,11 +207,11 @@ __device__ __forceinline__ void dig_mma(uint32_t d, uint64_t a, uint64_t b, uint
       : "memory");
 }
 
-// The products of one stage: nk16 groups of 16 K values; A: seven digit tiles,
+// The products of one stage: nk16 groups of 16 K values; A: D digit tiles,
 // `astep` bytes apart, of 128 rows (those beyond the rows in use may hold
-// anything: their accumulators are not read), B: seven of NB rows one after
+// anything: their accumulators are not read), B: D of NB rows one after
 // another.  first: the accumulators start at zero.  One thread.
-template <int NB>
+template <int NB, int D>
 __device__ __forceinline__ void dig_issue(uint32_t tmem, uint32_t a, uint32_t astep, uint32_t b, int nk16, bool first) {
   constexpr int PER = 256 / NB;  // digit blocks an instruction can take
   // the address field (16-byte units) is the only one that changes
@@ -176,11 +222,11 @@ __device__ __forceinline__ void dig_issue(uint32_t tmem, uint32_t a, uint32_t as
   uint32_t acc = first ? 0u : 1u;
   for (int ks = 0; ks < nk16; ++ks) {
 #pragma unroll
-    for (int i = 0; i < DIG; ++i) {
+    for (int i = 0; i < D; ++i) {
       const uint64_t da = ((uint64_t)dhi_a << 32) | (la + i * as);
 #pragma unroll
-      for (int j = 0; j < DIG - i; j += PER) {
-        const int nb = (DIG - i - j) < PER ? DIG - i - j : PER;
+      for (int j = 0; j < D - i; j += PER) {
+        const int nb = (D - i - j) < PER ? D - i - j : PER;
         const uint64_t db = ((uint64_t)dhi_b << 32) | (lb + j * (NB * 8));
         dig_mma(tmem + (i + j) * NB, da, db, dig_idesc(nb * NB), i == 0 ? acc : 1u);
       }
@@ -191,13 +237,13 @@ __device__ __forceinline__ void dig_issue(uint32_t tmem, uint32_t a, uint32_t as
   }
 }
 
-// The seven order sums of four neighbouring columns for this thread's lane
+// The order sums of four neighbouring columns for this thread's lane
 // (tensor-memory row).
-template <int NB>
-__device__ __forceinline__ void dig_sums4(uint32_t taddr, int (&a)[4][DIG]) {
-  uint32_t r[DIG][4];
+template <int NB, int D>
+__device__ __forceinline__ void dig_sums4(uint32_t taddr, int (&a)[4][D]) {
+  uint32_t r[D][4];
 #pragma unroll
-  for (int s = 0; s < DIG; ++s)
+  for (int s = 0; s < D; ++s)
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r[s][0]), "=r"(r[s][1]), "=r"(r[s][2]), "=r"(r[s][3])
                  : "r"(taddr + s * NB));
@@ -205,18 +251,30 @@ __device__ __forceinline__ void dig_sums4(uint32_t taddr, int (&a)[4][DIG]) {
 #pragma unroll
   for (int c = 0; c < 4; ++c)
 #pragma unroll
-    for (int s = 0; s < DIG; ++s) a[c][s] = __float2int_rn(__uint_as_float(r[s][c]));
+    for (int s = 0; s < D; ++s) a[c][s] = __float2int_rn(__uint_as_float(r[s][c]));
 }
 
 // Joined exactly: value = hi 2^32 + lo in units of 256^6 of the integer product.
 template <int NB>
 __device__ __forceinline__ void dig_drain4(uint32_t taddr, long long (&hi)[4], long long (&lo)[4]) {
   int a[4][DIG];
-  dig_sums4<NB>(taddr, a);
+  dig_sums4<NB, DIG>(taddr, a);
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     hi[c] = (long long)a[c][0] * 65536 + (a[c][1] * 256 + a[c][2]);
     lo[c] = (long long)a[c][3] * 16777216 + ((long long)a[c][4] * 65536 + ((long long)a[c][5] * 256 + a[c][6]));
+  }
+}
+
+// The same of eight digits, in units of 256^7.
+template <int NB>
+__device__ __forceinline__ void dig8_drain4(uint32_t taddr, long long (&hi)[4], long long (&lo)[4]) {
+  int a[4][DIG8];
+  dig_sums4<NB, DIG8>(taddr, a);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    hi[c] = (long long)a[c][0] * 16777216 + ((long long)a[c][1] * 65536 + ((long long)a[c][2] * 256 + a[c][3]));
+    lo[c] = (long long)a[c][4] * 16777216 + ((long long)a[c][5] * 65536 + ((long long)a[c][6] * 256 + a[c][7]));
   }
 }
 
@@ -226,7 +284,7 @@ __device__ __forceinline__ void dig_drain4(uint32_t taddr, long long (&hi)[4], l
 template <int NB>
 __device__ __forceinline__ void dig_join4(uint32_t taddr, long long (&t)[4]) {
   int a[4][DIG];
-  dig_sums4<NB>(taddr, a);
+  dig_sums4<NB, DIG>(taddr, a);
 #pragma unroll
   for (int c = 0; c < 4; ++c)
     t[c] = ((long long)(a[c][0] * 256 + a[c][1]) << 35) + (long long)a[c][2] * (1 << 27) + (long long)a[c][3] * (1 << 19) +
@@ -255,10 +313,19 @@ __device__ __forceinline__ double dig_value(long long t, int e, int f) {
   return __hiloint2double((int)(hi | (s & 0x80000000u)), (int)lo);
 }
 
-// The same for sums over several windows (|hi| < 2^62, |lo| < 2^63), in FP64.
+// The same for D digits' sums over several windows (|hi| < 2^62, |lo| < 2^63), in
+// FP64.
+template <int D>
 __device__ __forceinline__ double dig_value_sum(long long hi, long long lo, int e, int f) {
   if (e >= 0x7ff || f >= 0x7ff) return __longlong_as_double(0x7ff8000000000000LL);
-  return scalbn((double)hi * 4294967296.0 + (double)lo, e + f - 2104);
+  return scalbn((double)hi * 4294967296.0 + (double)lo, e + f - (D == DIG8 ? 2112 : 2104));
+}
+
+// Eight digits' sums over at most 1,024 values (below 2^78 units), by integer
+// operations; e and f as dig_value takes them.
+__device__ __forceinline__ double dig8_value_sum(long long hi, long long lo, int e, int f) {
+  hi += lo >> 32;
+  return dig_value((long long)(((unsigned long long)hi << 16) | ((uint32_t)lo >> 16)), e + 3, f);
 }
 
 // Tensor memory and the completion barrier of a CTA.  All threads call; every
@@ -305,11 +372,11 @@ __device__ __forceinline__ void dig_publish() {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
 }
-template <int NB>
+template <int NB, int D = DIG>
 __device__ __forceinline__ void dig_launch(const DigCta& c, uint32_t a, uint32_t astep, uint32_t b, int nk16, bool first) {
   if (threadIdx.x == DIG_ISSUER) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    dig_issue<NB>(c.tmem, a, astep, b, nk16, first);
+    dig_issue<NB, D>(c.tmem, a, astep, b, nk16, first);
     mma_commit(c.bar);
   }
 }
@@ -319,6 +386,27 @@ __device__ __forceinline__ void dig_wait(DigCta& c, int* abort) {
   if (!mbar_wait(c.bar, c.phase, *reinterpret_cast<volatile int*>(abort) ? 1u : DIG_POLLS)) atomicOr(abort, 1);
   c.phase ^= 1;
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
+
+// columns of B per chunk: a multiple of 16, at most 64 (seven blocks of
+// accumulators in tensor memory), the chunks as even as can be
+inline int chunk_cols(int n) {
+  const int c = (n + 63) / 64;
+  return ((n + c - 1) / c + 15) / 16 * 16;
+}
+
+// dynamic shared memory a CTA can have beside 3 KB of static
+constexpr size_t DIG_SMEM_MAX = 232448 - 3200;
+
+inline int sm_count() {
+  int dev = 0, n = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+  return n;
+}
+
+template <class K> void dig_opt_in(K k, size_t smem) {
+  cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
 }  // namespace

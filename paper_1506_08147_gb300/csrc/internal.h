@@ -35,8 +35,8 @@ struct BatchShape {
   // FFT kernels specialised for the line lengths at compile time
   int uni_nx = 0, uni_ny = 0, uni_nz = 0;
   bool ng_mult4 = true;  // every element's N_g is a multiple of 4 (16-byte columns)
-  // FP64 wave of the mixed form: Gram products in double-float arithmetic
-  // (FP32 pairs) instead of on the FP64 pipe
+  // FP64 wave of the mixed form: transforms and reductions in double-float
+  // arithmetic (FP32 pairs) instead of on the FP64 pipe
   bool dfloat = false;
   // 128-row tiles per CTA of the FP32 block update (tsmm_rows_kernel); a
   // launch shape only (each output's arithmetic is the same), tuned per
@@ -109,6 +109,13 @@ template <class real>
 void launch_gram(const Batch<real>& b, const GramJob<real>& job, double* partial, size_t partial_cap,
                  cudaStream_t st);
 
+// fp64_tensor.cu: the FP64 stage's Gram products and block updates on the tensor
+// cores by exact digit splitting
+size_t gram_dig_ints(const GramJob<double>& job, int ca, int cb, int nel);
+void launch_gram_dig(const Batch<double>& b, const GramJob<double>& job, double* partial, size_t pstride, int kchunk,
+                     int nchunk, int ca, int cb, int* exps, cudaStream_t st);
+void init_fp64_tensor_kernels();
+
 // Tall-skinny update out = alpha * sum_i in_i Y_i + beta * out, Y in FP64.
 enum { Y_RR = 0, Y_GXW = 1, Y_PTR = 2 };
 template <class real> struct TsmmJob {
@@ -133,6 +140,8 @@ template <class real> struct TsmmJob {
 template <class real>
 void launch_tsmm(const Batch<real>& b, const TsmmJob<real>& job, cudaStream_t st);
 void init_blas_kernels();
+// false where the job has more columns than the kernel takes
+bool launch_update_dig(const Batch<double>& b, const TsmmJob<double>& job, cudaStream_t st);
 
 // Residual R = HX - X diag(theta) into W, with per-column partial sums.
 template <class real>

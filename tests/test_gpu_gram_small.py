@@ -1,6 +1,5 @@
-"""FP64 Gram products of narrow blocks (csrc/blas.cu, gram48d_kernel): the
-widths at which the number of row groups of a CTA changes (tiles of 1, 2, 3, 4,
-5, 6, 8, 9 and 12 threads a side), on grids whose rows do not fill the chunks."""
+"""FP64 Gram products of narrow blocks (csrc/fp64_tensor.cu) at
+many widths, on grids whose rows do not fill the chunks."""
 
 import numpy as np
 import pytest
