@@ -221,6 +221,9 @@ __global__ void __launch_bounds__(144) gram48_kernel(const ElemDev<float>* __res
     for (int j = 0; j < 4; ++j) out[(ty * 4 + i) * TILE + tx * 4 + j] = (double)chi[i][j] + (double)clo[i][j];
 }
 
+// Partial sums added in the chunks' order, 16 CTAs per tile (one CTA per tile
+// left a step of few elements 0.27 ms in this kernel).
+// grid: (pairs and tiles, 16, nel).
 template <class real>
 __global__ void gram_reduce_kernel(const ElemDev<real>* __restrict__ elems, GramJob<real> job,
                                    const double* __restrict__ partial, size_t pstride, int nchunk,
@@ -246,10 +249,11 @@ __global__ void gram_reduce_kernel(const ElemDev<real>* __restrict__ elems, Gram
   }
   const double* base = partial + blockIdx.z * pstride + (size_t)blockIdx.x * (TILE * TILE);
   const size_t cstride = (size_t)gridDim.x * (TILE * TILE);
-  for (int i = threadIdx.x; i < TILE * TILE; i += blockDim.x) {
+  for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < TILE * TILE; i += gridDim.y * blockDim.x) {
     const int r = i / TILE, c = i - r * TILE;
     if (a0 + r >= ca || b0 + c >= cb) continue;
     double s = 0.0;
+#pragma unroll 8
     for (int ch = 0; ch < nchunk; ++ch) s += base[ch * cstride + i];
     const int orow = job.brow[pair] * ca + a0 + r;
     const int ocol = job.bcol[pair] * cb + b0 + c;
@@ -608,38 +612,60 @@ __global__ void __launch_bounds__(256) rnorm_kernel(const ElemDev<real>* __restr
   }
 }
 
+// Residual norms, kinetic energies, convergence.  One CTA per element; a thread
+// takes one of a column's four sums, or an eighth of its projector sum (with a
+// thread per column the chain of FP64 operations took 64 us at m = 48,
+// MEASURED_PR).
+constexpr int PR_COLS = 64, PR_PARTS = 8;
+
 template <class real>
-__global__ void post_residual_kernel(const ElemDev<real>* __restrict__ elems, int nchunk, int maxit) {
+__global__ void __launch_bounds__(PR_COLS * (4 + PR_PARTS))
+    post_residual_kernel(const ElemDev<real>* __restrict__ elems, int nchunk, int maxit) {
   const ElemDev<real>& e = elems[blockIdx.z];
   if (!e.state[ST_ACTIVE]) return;
-  __shared__ double smax[256];
-  __shared__ int sbad[256];
-  double mx = 0.0;
-  int bad = 0;
-  for (int j = threadIdx.x; j < e.m; j += blockDim.x) {
-    double s[4] = {0, 0, 0, 0};
-    for (int c = 0; c < nchunk; ++c)
-      for (int q = 0; q < 4; ++q) s[q] += e.rpart[((size_t)j * nchunk + c) * 4 + q];
-    double nl = 0.0;
-    for (int p = 0; p < e.n_proj; ++p) {
-      const double c = (double)e.Ccoef[p + (size_t)j * e.n_proj];
-      nl += e.p_gamma[p] * c * c;
-    }
-    const double res = sqrt(s[0] / s[1]);
-    e.res[j] = res;
-    // x.Hx was taken with H - sigma I
-    e.tkin[j] = (s[2] + e.sigma[0] * s[1] - s[3] - nl) / s[1];
-    if (!isfinite(res)) bad = 1;
-    if (j < e.J) mx = fmax(mx, res);
-  }
-  smax[threadIdx.x] = mx;
-  sbad[threadIdx.x] = bad;
-  __syncthreads();
+  __shared__ double ss[4][PR_COLS], sn[PR_PARTS][PR_COLS];
+  __shared__ unsigned long long smx;
+  __shared__ int sbad;
+  const int col = threadIdx.x & (PR_COLS - 1), part = threadIdx.x / PR_COLS;
   if (threadIdx.x == 0) {
-    for (int t = 1; t < blockDim.x; ++t) {
-      mx = fmax(mx, smax[t]);
-      bad |= sbad[t];
+    smx = 0ull;
+    sbad = 0;
+  }
+  for (int j0 = 0; j0 < e.m; j0 += PR_COLS) {
+    const int j = j0 + col;
+    if (j < e.m) {
+      double s = 0.0;
+      if (part < 4) {
+#pragma unroll 8
+        for (int c = 0; c < nchunk; ++c) s += e.rpart[((size_t)j * nchunk + c) * 4 + part];
+        ss[part][col] = s;
+      } else {
+#pragma unroll 4
+        for (int p = part - 4; p < e.n_proj; p += PR_PARTS) {
+          const double c = (double)e.Ccoef[p + (size_t)j * e.n_proj];
+          s += e.p_gamma[p] * c * c;
+        }
+        sn[part - 4][col] = s;
+      }
     }
+    __syncthreads();
+    if (part == 0 && j < e.m) {
+      double nl = 0.0;
+#pragma unroll
+      for (int p = 0; p < PR_PARTS; ++p) nl += sn[p][col];
+      const double res = sqrt(ss[0][col] / ss[1][col]);
+      e.res[j] = res;
+      // x.Hx was taken with H - sigma I
+      e.tkin[j] = (ss[2][col] + e.sigma[0] * ss[1][col] - ss[3][col] - nl) / ss[1][col];
+      if (!isfinite(res)) sbad = 1;
+      // (non-negative numbers compare as their bits)
+      else if (j < e.J) atomicMax(&smx, (unsigned long long)__double_as_longlong(res));
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    const double mx = __longlong_as_double((long long)smx);
+    const int bad = sbad;
     int* st = e.state;
     if (bad) {
       st[ST_ERROR] |= ERR_NONFINITE;
@@ -791,7 +817,7 @@ void launch_gram(const Batch<real>& b, const GramJob<real>& job, double* partial
     gram_kernel<real><<<dim3(nchunk, ny, s.nel), 256, 0, st>>>(b.d_elems, job, partial, pstride, kchunk,
                                                                tiles_a, tiles_b);
   }
-  gram_reduce_kernel<real><<<dim3(ny, 1, s.nel), 256, 0, st>>>(b.d_elems, job, partial, pstride, nchunk,
+  gram_reduce_kernel<real><<<dim3(ny, 16, s.nel), 256, 0, st>>>(b.d_elems, job, partial, pstride, nchunk,
                                                                tiles_a, tiles_b);
 }
 
@@ -827,7 +853,7 @@ void launch_residual(const Batch<real>& b, int nchunk, cudaStream_t st) {
 
 template <class real>
 void launch_post_residual(const Batch<real>& b, int nchunk, int maxit, cudaStream_t st) {
-  post_residual_kernel<real><<<dim3(1, 1, b.s.nel), 256, 0, st>>>(b.d_elems, nchunk, maxit);
+  post_residual_kernel<real><<<dim3(1, 1, b.s.nel), PR_COLS * (4 + PR_PARTS), 0, st>>>(b.d_elems, nchunk, maxit);
 }
 
 void launch_rnorm(const Batch<double>& b, int nchunk, cudaStream_t st) {
