@@ -239,7 +239,6 @@ bool launch_tf32_update(const Batch<float>& b, const TsmmJob<float>& job, const 
 bool launch_tf32_gram(const Batch<float>& b, const void* d_maps, int mode, double* partial, size_t partial_cap,
                       uint32_t polls, cudaStream_t st);
 
-// alb.cu
 // One product of the FP64 orthonormalisation for one element: the Gram
 // out = A^T A (J x J) or the update out = A Y (rows x J); column-major.
 struct OrthoTask {
@@ -249,12 +248,12 @@ struct OrthoTask {
   int rows, J;
   int K;            // columns of a in an update task (0: J)
 };
-constexpr int ORTHO_CHUNK = 1024;  // rows per CTA of the Gram
+// Both in fp64_tensor.cu; *err is set when a bounded device wait ran out, and at
+// most 1,024 columns are taken.  ortho_partial_doubles: the Gram's scratch.
 size_t ortho_partial_doubles(int ntask, int max_rows, int max_J);
-void launch_ortho_gram(const OrthoTask* d_tasks, int ntask, int max_rows, int max_J, double* partial,
+void launch_ortho_gram(const OrthoTask* d_tasks, int ntask, int max_rows, int max_J, double* partial, int* err,
                        cudaStream_t st);
-// the K x 32 Y columns of a CTA are staged in shared memory (K <= 900)
-void launch_ortho_apply(const OrthoTask* d_tasks, int ntask, int max_rows, int max_J, int max_K, cudaStream_t st);
+void launch_ortho_apply(const OrthoTask* d_tasks, int ntask, int max_rows, int max_J, int* err, cudaStream_t st);
 template <class real>
 void launch_restrict(const real* x, int ng, int nx, int ny, const int* lo, const int* hi, int J, double* out,
                      cudaStream_t st);

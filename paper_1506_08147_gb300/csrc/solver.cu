@@ -1383,6 +1383,7 @@ dgdft_status orthonormalise(dgdft_alb_ctx* ctx, Wave<double>& w, const std::vect
     Kmax = std::max(Kmax, Ks[q]);
     nemax = std::max(nemax, (size_t)ctx->el[w.ids[idx[q]]].ne());
   }
+  if (Kmax > 1024) return ctx->fail(DGDFT_ENOMEM, "orthonormalisation: more than 1,024 columns");
   const size_t jj = (size_t)Jmax * Jmax, kk = (size_t)Kmax * Kmax;
   // per element: phi_t (ne x K), U (ne x J), G (K x K), G2 (J x J), Y1
   // (K x J), Y2 (J x J), I (K x K), diag(1..J) (J x J), theta, Rayleigh-Ritz
@@ -1419,11 +1420,12 @@ dgdft_status orthonormalise(dgdft_alb_ctx* ctx, Wave<double>& w, const std::vect
     z.work = (double*)a.take(sizeof(double) * rr_work_doubles(Kmax, Kmax));
   }
   double* chk = (double*)a.take(sizeof(double) * nq);
+  int* terr = (int*)a.take(sizeof(int));  // a bounded device wait ran out
   double* part = (double*)a.take(sizeof(double) * npart);
   RRTask* dt = (RRTask*)a.take(2 * nq * sizeof(RRTask));  // [0, nq): first pass, [nq, 2nq): second
   // [0, nq): Gram of Phi~, then U = Phi~ Y1, Gram of U, out = U Y2
   OrthoTask* ot = (OrthoTask*)a.take(4 * nq * sizeof(OrthoTask));
-  if (!chk || !dt || !ot || !part || !sl.back().work) return ctx->fail(DGDFT_ENOMEM, "orthonormalisation scratch");
+  if (!chk || !terr || !dt || !ot || !part || !sl.back().work) return ctx->fail(DGDFT_ENOMEM, "orthonormalisation scratch");
   std::vector<double> hm((kk + jj) * nq, 0.0);
   std::vector<RRTask> ht(2 * nq);
   std::vector<OrthoTask> hot(4 * nq);
@@ -1465,22 +1467,26 @@ dgdft_status orthonormalise(dgdft_alb_ctx* ctx, Wave<double>& w, const std::vect
     const dgdft_element_desc& d = eh.d;
     launch_restrict<double>(xs[q], eh.ng(), d.nx, d.ny, d.e_lo, d.e_hi, Ks[q], sl[q].phit, st);
   }
-  launch_ortho_gram(ot, nqi, nem, Kmax, part, st);
+  CK(cudaMemsetAsync(terr, 0, sizeof(int), st));
+  launch_ortho_gram(ot, nqi, nem, Kmax, part, terr, st);
   launch_rr(dt, nqi, st, Kmax, Jmax);
   // U = Phi~ Y1 and its Gram, second Rayleigh-Ritz launch
-  launch_ortho_apply(ot + nq, nqi, nem, Jmax, Kmax, st);
-  launch_ortho_gram(ot + 2 * nq, nqi, nem, Jmax, part, st);
+  launch_ortho_apply(ot + nq, nqi, nem, Jmax, terr, st);
+  launch_ortho_gram(ot + 2 * nq, nqi, nem, Jmax, part, terr, st);
   launch_rr(dt + nq, nqi, st, Jmax, Jmax);
-  launch_ortho_apply(ot + 3 * nq, nqi, nem, Jmax, Jmax, st);
+  launch_ortho_apply(ot + 3 * nq, nqi, nem, Jmax, terr, st);
   for (size_t q = 0; q < nq; ++q) {
     const ElemHost& eh = ctx->el[w.ids[idx[q]]];
     launch_scale(out[q], (size_t)eh.ne() * Js[q], 1.0 / std::sqrt(eh.dv()), st);
     CK(cudaMemcpyAsync(chk + q, sl[q].th, sizeof(double), cudaMemcpyDeviceToDevice, st));
   }
   std::vector<double> hchk(nq);
+  int herr = 0;
   CK(cudaMemcpyAsync(hchk.data(), chk, sizeof(double) * nq, cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(&herr, terr, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   CK(cudaGetLastError());
+  if (herr) return ctx->fail(DGDFT_ETIMEOUT, "orthonormalisation: a bounded device wait ran out");
   for (size_t q = 0; q < nq; ++q) rank_ok[q] = std::isfinite(hchk[q]) ? 1 : 0;
   return DGDFT_OK;
 }
