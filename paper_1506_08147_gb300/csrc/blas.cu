@@ -26,15 +26,33 @@ __device__ __forceinline__ int ld_of(const ElemDev<real>& e, const BRef<real>& r
   return r.ptr ? (ld_in > 0 ? ld_in : rows) : e.ng;
 }
 
-// grid: (nchunk, npairs * tiles_a * tiles_b, nel); block 256 = 16 x 16.
-template <class real>
-__global__ void __launch_bounds__(256) gram_kernel(const ElemDev<real>* __restrict__ elems,
-                                                   GramJob<real> job, double* __restrict__ partial,
-                                                   size_t pstride, int kchunk, int tiles_a,
-                                                   int tiles_b) {
-  __shared__ real As[KS][TILE + 4];
-  __shared__ real Bs[KS][TILE + 4];
-  const ElemDev<real>& e = elems[blockIdx.z];
+constexpr int GK = 32;  // rows per stage of the FP32 Gram kernels
+
+// a stage holds columns, rows contiguous; the 16-byte chunks of a column are
+// swizzled by column group, so that a warp's column groups hit distinct banks
+__device__ __forceinline__ int g48_off(int c, int r) {
+  return c * GK + ((((r >> 2) ^ ((c >> 2) & 7)) << 2) | (r & 3));
+}
+
+// FP32 Gram products of blocks of more than 48 columns: ceil(m / 64) tiles of equal
+// width (a multiple of 4, at most 64) a side, 4 x 4 outputs a thread, so that no
+// thread works on columns past m (64-wide tiles did 1.8 times the work at m = 144,
+// 2.8 at m = 72).  The next 32 rows are on their way (16-byte
+// cp.async) while this stage's products run.  A step of two elements of 144
+// columns: 30 -> 19.4 ms in this kernel; six boxes of 32 to 104: 13.3 -> 8.8.  (Two
+// FMAs to an instruction, for even and odd rows: 19.7 and 10.1, at 128 registers.)
+// grid: (nchunk, npairs * tiles_a * tiles_b, nel); block 256.
+__host__ __device__ __forceinline__ int gram_tile(int m) {
+  const int nt = (m + TILE - 1) / TILE;
+  return ((m + nt - 1) / nt + 3) & ~3;
+}
+
+__global__ void __launch_bounds__(256, 3) gram_kernel(const ElemDev<float>* __restrict__ elems, GramJob<float> job,
+                                                      double* __restrict__ partial, size_t pstride, int kchunk,
+                                                      int tiles_a, int tiles_b) {
+  __shared__ __align__(16) float As[2][TILE * KS];
+  __shared__ __align__(16) float Bs[2][TILE * KS];
+  const ElemDev<float>& e = elems[blockIdx.z];
   if (!e.state[ST_ACTIVE]) return;
   const int ntile = tiles_a * tiles_b;
   const int pair = blockIdx.y / ntile;
@@ -44,67 +62,94 @@ __global__ void __launch_bounds__(256) gram_kernel(const ElemDev<real>* __restri
   const int ca = job.ncols_a > 0 ? job.ncols_a : e.m;
   const int cb = job.ncols_b > 0 ? job.ncols_b : e.m;
   const int rows = job.rows > 0 ? job.rows : e.ng;
-  const int a0 = ta * TILE, b0 = tb * TILE;
+  const int wa = gram_tile(ca), wb = gram_tile(cb), a0 = ta * wa, b0 = tb * wb;
   if (a0 >= ca || b0 >= cb) return;
-  const real* A = resolve(e, job.a[pair]);
-  const real* B = resolve(e, job.b[pair]);
   const int lda = ld_of(e, job.a[pair], job.ld_in, rows);
   const int ldb = ld_of(e, job.b[pair], job.ld_in, rows);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const float* A = resolve(e, job.a[pair]) + (size_t)a0 * lda;
+  const float* B = resolve(e, job.b[pair]) + (size_t)b0 * ldb;
+  const int na = min(wa, ca - a0), nb = min(wb, cb - b0);
+  const int ndx = wb / 4, ndy = wa / 4;  // threads along the columns of B and of A
+  const int tx = threadIdx.x % ndx, ty = threadIdx.x / ndx;
+  const bool work = ty < ndy;
   const int k_beg = blockIdx.x * kchunk;
   const int k_end = min(rows, k_beg + kchunk);
-  real acc[4][4];
-  // FP32: each KS-row step is summed in FP32 and folded into a compensated
+  float acc[4][4];
+  // each KS-row step is summed in FP32 and folded into a compensated
   // (hi, lo) pair, so rounding does not grow with the chunk length (the
   // Gram entries carry residual information ~1e-6 of their size)
-  real chi[4][4], clo[4][4];
+  float chi[4][4], clo[4][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = chi[i][j] = clo[i][j] = 0;
-  for (int k0 = k_beg; k0 < k_end; k0 += KS) {
-    for (int i = threadIdx.x; i < KS * TILE; i += blockDim.x) {
-      const int c = i / KS, r = i - c * KS;
-      const int k = k0 + r;
-      const bool kin = k < k_end;
-      As[r][c] = (kin && a0 + c < ca) ? A[(size_t)(a0 + c) * lda + k] : (real)0;
-      Bs[r][c] = (kin && b0 + c < cb) ? B[(size_t)(b0 + c) * ldb + k] : (real)0;
+    for (int j = 0; j < 4; ++j) acc[i][j] = chi[i][j] = clo[i][j] = 0.f;
+  const bool vec = ((lda | ldb | k_beg) & 3) == 0 && ((((uintptr_t)A) | ((uintptr_t)B)) & 15) == 0;
+  // four rows of a column at a time
+  auto load1 = [&](float* dst, const float* src, int ld, int n, int w, int k0) {
+#pragma unroll
+    for (int q = 0; q < TILE * KS / 4 / 256; ++q) {
+      const int i = threadIdx.x + 256 * q, c = i >> 3, r = 4 * (i & 7);
+      if (c >= w) break;
+      const int nv = c < n ? max(0, min(4, k_end - k0 - r)) : 0;
+      const float* g = nv ? src + (size_t)c * ld + k0 + r : src;
+      float* d = dst + g48_off(c, r);
+      if (vec) {
+        cp_async16(d, g, 4 * nv);
+      } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) cp_async4(d + u, u < nv ? g + u : src, u < nv ? 4 : 0);
+      }
     }
-    __syncthreads();
-#pragma unroll 8
-    for (int r = 0; r < KS; ++r) {
-      real av[4], bv[4];
+  };
+  auto load = [&](int s, int k0) {
+    load1(As[s], A, lda, na, wa, k0);
+    load1(Bs[s], B, ldb, nb, wb, k0);
+    cp_async_commit();
+  };
+  load(0, k_beg);
+  int s = 0;
+  for (int k0 = k_beg; k0 < k_end; k0 += KS, s ^= 1) {
+    cp_async_wait<0>();
+    __syncthreads();  // this stage has arrived, the other one is no longer read
+    if (k0 + KS < k_end) load(s ^ 1, k0 + KS);
+    if (work) {
+#pragma unroll 2
+      for (int r = 0; r < KS; r += 4) {
+        float4 b4[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) av[i] = As[r][ty * 4 + i];
+        for (int j = 0; j < 4; ++j) b4[j] = *reinterpret_cast<const float4*>(&Bs[s][g48_off(tx * 4 + j, r)]);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) bv[j] = Bs[r][tx * 4 + j];
+        for (int i = 0; i < 4; ++i) {
+          const float4 a4 = *reinterpret_cast<const float4*>(&As[s][g48_off(ty * 4 + i, r)]);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] += av[i] * bv[j];
-    }
-    __syncthreads();
-    if constexpr (sizeof(real) == sizeof(float)) {
+          for (int j = 0; j < 4; ++j) {
+            acc[i][j] = fmaf(a4.x, b4[j].x, acc[i][j]);
+            acc[i][j] = fmaf(a4.y, b4[j].y, acc[i][j]);
+            acc[i][j] = fmaf(a4.z, b4[j].z, acc[i][j]);
+            acc[i][j] = fmaf(a4.w, b4[j].w, acc[i][j]);
+          }
+        }
+      }
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           // Knuth's two-sum of chi + acc: exact error term into clo
-          const real sum = chi[i][j] + acc[i][j];
-          const real bp = sum - chi[i][j];
+          const float sum = chi[i][j] + acc[i][j];
+          const float bp = sum - chi[i][j];
           clo[i][j] += (chi[i][j] - (sum - bp)) + (acc[i][j] - bp);
           chi[i][j] = sum;
-          acc[i][j] = 0;
+          acc[i][j] = 0.f;
         }
     }
   }
+  if (!work) return;
   double* out = partial + blockIdx.z * pstride +
                 ((size_t)blockIdx.x * gridDim.y + blockIdx.y) * (TILE * TILE);
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-      out[(ty * 4 + i) * TILE + tx * 4 + j] = (double)acc[i][j] + (double)chi[i][j] + (double)clo[i][j];
+    for (int j = 0; j < 4; ++j) out[(ty * 4 + i) * TILE + tx * 4 + j] = (double)chi[i][j] + (double)clo[i][j];
 }
 
 // FP32 Gram products for blocks of at most 48 columns (the LOBPCG pencil at
@@ -118,11 +163,6 @@ __global__ void __launch_bounds__(256) gram_kernel(const ElemDev<real>* __restri
 // compensated pair.  Partials use gram_kernel's 64 x 64 layout.
 // grid: (npairs, nchunk, nel); block 144.
 constexpr int G48 = 48;
-constexpr int GK = 32;  // rows per stage
-
-__device__ __forceinline__ int g48_off(int c, int r) {
-  return c * GK + ((((r >> 2) ^ ((c >> 2) & 7)) << 2) | (r & 3));
-}
 
 __global__ void __launch_bounds__(144) gram48_kernel(const ElemDev<float>* __restrict__ elems,
                                                       GramJob<float> job, double* __restrict__ partial,
@@ -237,7 +277,9 @@ __global__ void gram_reduce_kernel(const ElemDev<real>* __restrict__ elems, Gram
   if (job.needs_p[pair] && !e.state[ST_HAS_P]) return;
   const int ca = job.ncols_a > 0 ? job.ncols_a : e.m;
   const int cb = job.ncols_b > 0 ? job.ncols_b : e.m;
-  const int a0 = ta * TILE, b0 = tb * TILE;
+  // FP64 partials come in 64-column tiles, FP32 ones in tiles of equal width
+  constexpr bool f32 = std::is_same<real, float>::value;
+  const int wa = f32 ? gram_tile(ca) : TILE, wb = f32 ? gram_tile(cb) : TILE, a0 = ta * wa, b0 = tb * wb;
   if (a0 >= ca || b0 >= cb) return;
   double* out;
   int ld;
@@ -251,7 +293,7 @@ __global__ void gram_reduce_kernel(const ElemDev<real>* __restrict__ elems, Gram
   const size_t cstride = (size_t)gridDim.x * (TILE * TILE);
   for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < TILE * TILE; i += gridDim.y * blockDim.x) {
     const int r = i / TILE, c = i - r * TILE;
-    if (a0 + r >= ca || b0 + c >= cb) continue;
+    if (r >= wa || c >= wb || a0 + r >= ca || b0 + c >= cb) continue;
     double s = 0.0;
 #pragma unroll 8
     for (int ch = 0; ch < nchunk; ++ch) s += base[ch * cstride + i];
@@ -814,7 +856,7 @@ void launch_gram(const Batch<real>& b, const GramJob<real>& job, double* partial
   } else if (ca <= G48 && cb <= G48) {
     gram48_kernel<<<dim3(ny, nchunk, s.nel), 144, 0, st>>>(b.d_elems, job, partial, pstride, kchunk);
   } else {
-    gram_kernel<real><<<dim3(nchunk, ny, s.nel), 256, 0, st>>>(b.d_elems, job, partial, pstride, kchunk,
+    gram_kernel<<<dim3(nchunk, ny, s.nel), 256, 0, st>>>(b.d_elems, job, partial, pstride, kchunk,
                                                                tiles_a, tiles_b);
   }
   gram_reduce_kernel<real><<<dim3(ny, 16, s.nel), 256, 0, st>>>(b.d_elems, job, partial, pstride, nchunk,

@@ -437,8 +437,8 @@ template <class real> struct Wave {
         s.uni_nz = d0.nz;
       }
     }
-    // the refinement (FP64) stage of the mixed form takes its Gram products
-    // in double-float arithmetic; the plain FP64 solver stays on the FP64 pipe
+    // the refinement (FP64) stage of the mixed form takes its transforms and
+    // reductions in double-float arithmetic; the plain FP64 solver in FP64
     s.dfloat = std::is_same<real, double>::value && ctx->cfg.precision == DGDFT_PREC_MIXED;
     rnchunk = nchunk_rows(s.max_ng);
     const size_t pcap = (size_t)nel * gram_partial_doubles(s.max_ng, s.max_m);
