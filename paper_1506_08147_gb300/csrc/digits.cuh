@@ -322,10 +322,14 @@ __device__ __forceinline__ double dig_value_sum(long long hi, long long lo, int 
 }
 
 // Eight digits' sums over at most 1,024 values (below 2^78 units), by integer
-// operations; e and f as dig_value takes them.
+// operations; e and f as dig_value takes them.  The 63 leading bits are kept
+// wherever they lie (the 63 at fixed places would cut results well below the
+// largest product short).
 __device__ __forceinline__ double dig8_value_sum(long long hi, long long lo, int e, int f) {
   hi += lo >> 32;
-  return dig_value((long long)(((unsigned long long)hi << 16) | ((uint32_t)lo >> 16)), e + 3, f);
+  const int sh = min(__clzll(hi ^ (hi >> 63)) - 1, 32);  // at least 16
+  const unsigned long long t = ((unsigned long long)hi << sh) | ((unsigned long long)(uint32_t)lo >> (32 - sh));
+  return dig_value((long long)t, e + 19 - sh, f);
 }
 
 // Tensor memory and the completion barrier of a CTA.  All threads call; every
