@@ -260,6 +260,6 @@ void launch_restrict(const real* x, int ng, int nx, int ny, const int* lo, const
 template <class A, class B>
 void launch_convert(const A* in, B* out, size_t n, cudaStream_t st);
 void launch_scale(double* x, size_t n, double s, cudaStream_t st);
-// flag |= 1 when any of x[0..n) is not finite
-void launch_nonfinite(const double* x, size_t n, int* flag, cudaStream_t st);
+// dst = src, flag |= 1 when any of the n values is not finite
+void launch_copy_checked(const double* src, double* dst, size_t n, int* flag, cudaStream_t st);
 }  // namespace dgdft

@@ -154,6 +154,29 @@ struct dgdft_alb_ctx {
   // (grown when a call needs more)
   void* ortho_buf = nullptr;
   size_t ortho_cap = 0;
+  // page-locked staging of the small per-element copies (states, residuals,
+  // eigenvalues; a copy to pageable memory waits for itself, 10 us each) and
+  // the input check's flag; a context's calls are on one stream, and each
+  // waits for its copies before it returns
+  char* pin_buf = nullptr;
+  size_t pin_cap = 0;
+  int* d_flag = nullptr;
+  // nullptr when the memory cannot be had
+  char* pin(size_t bytes) {
+    if (bytes > pin_cap) {
+      if (pin_buf) cudaFreeHost(pin_buf);
+      pin_buf = nullptr;
+      pin_cap = 0;
+      const size_t cap = bytes + 65536;
+      if (cudaMallocHost((void**)&pin_buf, cap) != cudaSuccess) {
+        cudaGetLastError();
+        pin_buf = nullptr;
+        return nullptr;
+      }
+      pin_cap = cap;
+    }
+    return pin_buf;
+  }
   std::vector<int> cache_proj_version;
   ConvNet* net = nullptr;  // learned preconditioner, created on first use
   int wait_polls = 0;      // bounded device waits: polls before giving up (0: default)
@@ -830,18 +853,38 @@ template <class real> struct Wave {
       }
       h[i].tol = tol;
     }
-    CK(ctx_copy(ctx, d_elems, h.data(), sizeof(ElemDev<real>) * nel, cudaMemcpyHostToDevice));
+    const size_t eb = sizeof(ElemDev<real>) * nel, sb = sizeof(int) * STATE_WORDS;
+    char* p = ctx->pin(eb + sb * nel);
+    if (!p) return ctx->fail(DGDFT_ENOMEM, "page-locked staging");
+    std::memcpy(p, h.data(), eb);
+    std::memcpy(p + eb, h_state.data(), sb * nel);
+    CK(cudaMemcpyAsync(d_elems, p, eb, cudaMemcpyHostToDevice, ctx->stream));
     for (int i = 0; i < nel; ++i)
-      CK(ctx_copy(ctx, h[i].state, &h_state[(size_t)i * STATE_WORDS], sizeof(int) * STATE_WORDS,
-                    cudaMemcpyHostToDevice));
+      CK(cudaMemcpyAsync(h[i].state, p + eb + sb * i, sb, cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
     return DGDFT_OK;
   }
 
   dgdft_status read_states() {
-    for (size_t i = 0; i < ids.size(); ++i)
-      CK(cudaMemcpyAsync(&h_state[i * STATE_WORDS], h[i].state, sizeof(int) * STATE_WORDS,
-                         cudaMemcpyDeviceToHost, ctx->stream));
+    const size_t nel = ids.size(), sb = sizeof(int) * STATE_WORDS;
+    char* p = ctx->pin(sb * nel);
+    if (!p) return ctx->fail(DGDFT_ENOMEM, "page-locked staging");
+    for (size_t i = 0; i < nel; ++i)
+      CK(cudaMemcpyAsync(p + sb * i, h[i].state, sb, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
+    std::memcpy(h_state.data(), p, sb * nel);
+    return DGDFT_OK;
+  }
+
+  // the residuals of every element, max_m apart, in the page-locked staging
+  dgdft_status read_residuals(const double*& res) {
+    const size_t nel = ids.size(), ld = (size_t)batch.s.max_m;
+    double* p = (double*)ctx->pin(sizeof(double) * ld * nel);
+    if (!p) return ctx->fail(DGDFT_ENOMEM, "page-locked staging");
+    for (size_t i = 0; i < nel; ++i)
+      CK(cudaMemcpyAsync(p + ld * i, h[i].res, sizeof(double) * h[i].m, cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
+    res = p;
     return DGDFT_OK;
   }
 
@@ -1217,7 +1260,6 @@ template <class real> struct Wave {
     const int every = std::max(1, ctx->cfg.check_every);
     std::vector<std::vector<double>> hist(nel);
     std::vector<int> seen_restarts(nel, 0);
-    std::vector<double> resbuf;
     int launched = 0;
     dgdft_status rs = DGDFT_OK;
     int since_refresh = 0;
@@ -1249,6 +1291,8 @@ template <class real> struct Wave {
       }
       bool any = false;
       std::vector<double> active_res;  // read only with a stall window
+      const double* resp = nullptr;
+      if (stall_window > 0 && (rs = read_residuals(resp)) != DGDFT_OK) break;
       for (int i = 0; i < nel; ++i) {
         int* sw = &h_state[(size_t)i * STATE_WORDS];
         if (!sw[ST_ACTIVE]) continue;
@@ -1260,10 +1304,8 @@ template <class real> struct Wave {
             seen_restarts[i] = sw[ST_NRESTART];
             hist[i].clear();
           }
-          resbuf.resize(h[i].J);
-          ce = ctx_copy(ctx, resbuf.data(), h[i].res, sizeof(double) * h[i].J, cudaMemcpyDeviceToHost);
-          if (ce != cudaSuccess) break;
-          const double mx = *std::max_element(resbuf.begin(), resbuf.end());
+          const double* ri = resp + (size_t)i * batch.s.max_m;
+          const double mx = *std::max_element(ri, ri + h[i].J);
           hist[i].push_back(mx);
           active_res.push_back(mx);
           const size_t L = hist[i].size();
@@ -1335,11 +1377,9 @@ template <class real> struct Wave {
     CK(cudaGetLastError());
     if (res_out) {
       res_out->clear();
-      for (int i = 0; i < nel; ++i) {
-        std::vector<double> r(h[i].m);
-        CK(ctx_copy(ctx, r.data(), h[i].res, sizeof(double) * h[i].m, cudaMemcpyDeviceToHost));
-        res_out->insert(res_out->end(), r.begin(), r.end());
-      }
+      const double* r = nullptr;
+      if ((rs = read_residuals(r)) != DGDFT_OK) return rs;
+      for (int i = 0; i < nel; ++i) res_out->insert(res_out->end(), r + (size_t)i * batch.s.max_m, r + (size_t)i * batch.s.max_m + h[i].m);
     }
     return read_states();
   }
@@ -1548,15 +1588,21 @@ dgdft_status finish_wave(dgdft_alb_ctx* ctx, Wave<double>& w, int wave_idx, doub
     if (so != DGDFT_OK) return so;
   }
   // eigenvalues and residuals of every element to the host, one wait
+  const size_t ldp = (size_t)w.batch.s.max_m;
+  double* stage = (double*)ctx->pin(sizeof(double) * 2 * ldp * nel);
+  if (!stage) return ctx->fail(DGDFT_ENOMEM, "page-locked staging");
   for (size_t i = 0; i < nel; ++i) {
-    ElemHost& eh = ctx->el[w.ids[i]];
     const ElemDev<double>& E = w.h[i];
-    eh.eig.resize(E.J);
-    eh.resid.resize(E.J);
-    CK(cudaMemcpyAsync(eh.eig.data(), E.theta, sizeof(double) * E.J, cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaMemcpyAsync(eh.resid.data(), E.res, sizeof(double) * E.J, cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaMemcpyAsync(stage + 2 * ldp * i, E.theta, sizeof(double) * E.J, cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaMemcpyAsync(stage + 2 * ldp * i + ldp, E.res, sizeof(double) * E.J, cudaMemcpyDeviceToHost, ctx->stream));
   }
   CK(cudaStreamSynchronize(ctx->stream));
+  for (size_t i = 0; i < nel; ++i) {
+    ElemHost& eh = ctx->el[w.ids[i]];
+    const double* p = stage + 2 * ldp * i;
+    eh.eig.assign(p, p + w.h[i].J);
+    eh.resid.assign(p + ldp, p + ldp + w.h[i].J);
+  }
   for (size_t i = 0; i < nel; ++i) {
     ElemHost& eh = ctx->el[w.ids[i]];
     const ElemDev<double>& E = w.h[i];
@@ -1946,20 +1992,21 @@ static dgdft_status copy_resident(dgdft_alb_ctx* ctx, double*& dst, const double
       return ctx->fail(DGDFT_ENOMEM, "resident input allocation: " + cuda_err_string(e));
     }
   }
-  CK(ctx_copy(ctx, dst, src, sizeof(double) * n, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice));
-  if (on_device) {
-    int* flag = nullptr;
-    CK(cudaMalloc(&flag, sizeof(int)));
-    int h = 0;
-    cudaError_t e = ctx_copy(ctx, flag, &h, sizeof(int), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) {
-      launch_nonfinite(dst, n, flag, ctx->stream);
-      e = ctx_copy(ctx, &h, flag, sizeof(int), cudaMemcpyDeviceToHost);
-    }
-    cudaFree(flag);
-    if (e != cudaSuccess) return ctx->fail(DGDFT_ECUDA, "input check: " + cuda_err_string(e));
-    if (h) return ctx->fail(DGDFT_EINVAL, "non-finite input value");
+  if (!on_device) {
+    CK(ctx_copy(ctx, dst, src, sizeof(double) * n, cudaMemcpyHostToDevice));
+    return DGDFT_OK;
   }
+  // one kernel copies and checks (separate copies to and from pageable memory
+  // around a check made this 65 us a call)
+  if (!ctx->d_flag) CK(cudaMalloc(&ctx->d_flag, sizeof(int)));
+  int* h = (int*)ctx->pin(sizeof(int));
+  if (!h) return ctx->fail(DGDFT_ENOMEM, "page-locked staging");
+  CK(cudaMemsetAsync(ctx->d_flag, 0, sizeof(int), ctx->stream));
+  launch_copy_checked(src, dst, n, ctx->d_flag, ctx->stream);
+  CK(cudaGetLastError());
+  CK(cudaMemcpyAsync(h, ctx->d_flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  CK(cudaStreamSynchronize(ctx->stream));
+  if (*h) return ctx->fail(DGDFT_EINVAL, "non-finite input value");
   return DGDFT_OK;
 }
 
@@ -2074,9 +2121,10 @@ dgdft_status dgdft_alb_get_basis(dgdft_alb_ctx* ctx, int elem, double* phi, doub
   if (!eh.solved) return ctx->fail(DGDFT_ESTATE, "get_basis before solve");
   const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   const size_t J = eh.d.n_keep;
-  if (phi) CK(ctx_copy(ctx, phi, eh.d_phi, sizeof(double) * J * eh.ne(), k));
-  if (eig) CK(ctx_copy(ctx, eig, eh.d_eig, sizeof(double) * J, k));
-  if (resid) CK(ctx_copy(ctx, resid, eh.d_res, sizeof(double) * J, k));
+  if (phi) CK(cudaMemcpyAsync(phi, eh.d_phi, sizeof(double) * J * eh.ne(), k, ctx->stream));
+  if (eig) CK(cudaMemcpyAsync(eig, eh.d_eig, sizeof(double) * J, k, ctx->stream));
+  if (resid) CK(cudaMemcpyAsync(resid, eh.d_res, sizeof(double) * J, k, ctx->stream));
+  CK(cudaStreamSynchronize(ctx->stream));
   return DGDFT_OK;
 }
 
@@ -2087,6 +2135,8 @@ void dgdft_alb_destroy(dgdft_alb_ctx* ctx) {
   cudaSetDevice(ctx->device);
   ctx->drop_cache();
   if (ctx->ortho_buf) cudaFree(ctx->ortho_buf);
+  if (ctx->pin_buf) cudaFreeHost(ctx->pin_buf);
+  if (ctx->d_flag) cudaFree(ctx->d_flag);
   for (ElemHost& eh : ctx->el) eh.release();
   delete ctx->net;
   if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
