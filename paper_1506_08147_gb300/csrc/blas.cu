@@ -871,12 +871,19 @@ void launch_tsmm(const Batch<real>& b, const TsmmJob<real>& job, cudaStream_t st
     const size_t smem = tsmm_rows_smem(job.nin, nc);
     if (smem <= 160 * 1024) {
       const int rows = job.rows > 0 ? job.rows : s.max_ng;
-      // s.tsmm_tiles 128-row tiles per CTA (default 8, or the autotuner's
-      // choice): the Y staging (ktot x 48 coefficients per CTA) is amortised;
-      // 1.87 ms against 2.24 ms with two tiles on the 36-element monolayer
-      const int tpc = s.tsmm_tiles > 0 ? s.tsmm_tiles : 8;
+      // 128-row tiles per CTA: the autotuner's choice, or as few (at most
+      // eight) as leave every CTA resident at once.  More tiles amortise the Y
+      // staging (ktot x 48 coefficients per CTA), too few CTAs leave the SMs with
+      // four warps each, and a second round of CTAs is mostly empty: 960 tiles
+      // of one element take 154 us at eight, 86 at two, 92 at one; two elements
+      // 194 at eight, 150 at four; 36 elements 1.87 ms at eight, 2.22 at two.
+      const int nct = (nc + TS_CT - 1) / TS_CT, ntile = (rows + TS_TR - 1) / TS_TR;
+      const int slots = 152 * (int)std::min<size_t>(4, (227 * 1024) / (smem + 1024));
+      int tpc = s.tsmm_tiles;
+      if (tpc <= 0)
+        for (tpc = 1; tpc < 8 && (long long)((ntile + tpc - 1) / tpc) * nct * s.nel > slots;) ++tpc;
       const int gx = std::max(1, (rows + tpc * TS_TR - 1) / (tpc * TS_TR));
-      tsmm_rows_kernel<<<dim3(gx, (nc + TS_CT - 1) / TS_CT, s.nel), TS_THREADS, smem, st>>>(b.d_elems, job);
+      tsmm_rows_kernel<<<dim3(gx, nct, s.nel), TS_THREADS, smem, st>>>(b.d_elems, job);
       return;
     }
   }

@@ -40,8 +40,9 @@ struct BatchShape {
   bool dfloat = false;
   // 128-row tiles per CTA of the FP32 block update (tsmm_rows_kernel); a
   // launch shape only (each output's arithmetic is the same), tuned per
-  // batch shape when the context has an autotune cache
-  int tsmm_tiles = 8;
+  // batch shape when the context has an autotune cache, else (0) chosen by the
+  // launch
+  int tsmm_tiles = 0;
 };
 
 template <class real> struct Batch {
