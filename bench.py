@@ -208,9 +208,6 @@ def dg_load_inputs(B, d, dom):
         d.dgdft_dg_set_projectors(k, pid, rp, idx, val)
 
 
-DFLOAT_PEAK_TFLOPS = 7.85 * 152 * 2.07e9 * 2 / 1e12  # measured double-float FMA/clk/SM
-
-
 def dg_measure(B, dom, blocks, stream, steps, warmup, cap_bytes=0, dfloat=False, density=True):
     """Time the DG assembly (Eq. DGHamiltonian) of every element from the
     given device columns with CUDA events on the library's stream."""
@@ -235,11 +232,10 @@ def dg_measure(B, dom, blocks, stream, steps, warmup, cap_bytes=0, dfloat=False,
     flops = dg_flops_per_element(dom) * dom.n_elem
     achieved = flops / (ms / 1e3) / 1e12
     dominant = max(stage_ms, key=stage_ms.get)
-    if dfloat:
-        peak, src, kind = (DFLOAT_PEAK_TFLOPS, "double-float pairs: measured 7.85 FMA/clk/SM x 152 SMs x 2.07 GHz",
-                           "double-float SIMT")
-    else:
-        peak, src, kind = (FP64_PEAK_TFLOPS, "FP64 pipe: measured 1.91 FMA/clk/SM x 152 SMs x 2.07 GHz", "FP64 SIMT")
+    # both arithmetic options run FP64 products as 28 FP16 digit products on the
+    # tensor cores
+    peak, kind = peaks()[1] / 28, "FP64 by digit splitting, tcgen05"
+    src = "measured bf16_tflops / 28 digit products (MEASURED_PEAKS.json)"
     out = {"ms_per_assembly": round(ms, 3), "elements": dom.n_elem, "J": dom.J,
            "lgl_points": list(dom.nl), "blocks": nblk, "arith": "double-float" if dfloat else "fp64",
            "stage_ms": {k: round(v, 3) for k, v in stage_ms.items()}, "launches": launches,

@@ -49,10 +49,9 @@ dgdft_status dgdft_alb_gram(dgdft_alb_ctx* ctx, int ng, int p, int q, const doub
  * products Phi^T Psi), computed on caller blocks by the same kernels and
  * with the same precision choices as the solver for element `elem`, in the
  * stage `stage` selects: 0 the bulk stage (in DGDFT_PREC_MIXED the FP32
- * stage: tensor cores unless bulk_kernels = 1), 1 the FP64 stage (in
- * DGDFT_PREC_MIXED double-float products, FP32 pairs with exact products
- * and two-sum accumulation, ~2^-44 relative; plain FP64 in
- * DGDFT_PREC_FP64, where both stages are the same).  blocks holds
+ * stage: tensor cores unless bulk_kernels = 1), 1 the FP64 stage (FP64
+ * products, exact to 2^-60 of the columns' largest entries, in either
+ * precision mode; in DGDFT_PREC_FP64 both stages are the same).  blocks holds
  * six N_g x m column-major blocks one after another: X, W, P, H X, H W, H P
  * (m = n_compute; P and H P are ignored when has_p = 0).  With S = [X W P]:
  * a = (H S)^T S and b = S^T S, each 3m x 3m column-major, are returned in
@@ -69,7 +68,7 @@ dgdft_status dgdft_alb_lobpcg_gram(dgdft_alb_ctx* ctx, int elem, int stage, int 
  * paper's Phi C products), computed on caller blocks by the same kernels
  * and precision choices as the solver for element `elem` in stage `stage`
  * (0: the bulk stage, in DGDFT_PREC_MIXED the FP32 stage, tensor cores when
- * bulk_kernels = 2; 1: the FP64 stage, double-float in DGDFT_PREC_MIXED).
+ * bulk_kernels = 2; 1: the FP64 stage).
  * blocks holds six N_g x m column-major blocks: X, W, P, H X, H W, H P (P
  * and H P ignored when has_p = 0); y is the 3m x m column-major coefficient
  * block [Y_x; Y_w; Y_p] of a Rayleigh-Ritz step.  out receives three N_g x m

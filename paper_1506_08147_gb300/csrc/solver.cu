@@ -1000,9 +1000,9 @@ template <class real> struct Wave {
     g.out_id[1] = OUT_GRAM_B;
     for (int k = 0; k < 2; ++k) g.needs_p[k] = g.brow[k] = g.bcol[k] = 0;
     launch_gram<real>(batch, g, partial, partial_cap, st);
-    // double-float reduction in the FP32 stage and in the mixed form's
-    // FP64-accurate stage (its pencils carry the double-float Gram's ~2^-44
-    // rounding; the reduction's ~2^-46 adds nothing), FP64 otherwise
+    // double-float reduction (~2^-46) in the FP32 stage and in the mixed
+    // form's FP64-accurate stage, whose transforms are double-float too; FP64
+    // otherwise
     launch_rr(d_rr_init, batch.s.nel, st, batch.s.max_m, batch.s.max_m,
               std::is_same<real, float>::value || batch.s.dfloat);
     TsmmJob<real> t;
