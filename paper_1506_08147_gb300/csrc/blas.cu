@@ -541,8 +541,12 @@ size_t tsmm_rows_smem(int nin, int nc) {
   return sizeof(float) * ((size_t)nin * nc * TS_CT + 2 * (size_t)TS_TK * TS_TR);
 }
 
-// R = HX - X diag(theta) into W; partial sums (r.r, x.x, x.Hx, x.V x).
-template <class real>
+// R = HX - X diag(theta) into W; partial sums (r.r, x.x, x.Hx, x.V x).  PART 1:
+// only the sums that need no theta, 2: only R and r.r, for a check that first
+// needs the Rayleigh quotients (the FP64 pipe bounds the FP64 kernel, six
+// instructions a point: two full passes over 36 elements took 5.3 ms, the
+// two parts take 2.7).
+template <class real, int PART>
 __global__ void __launch_bounds__(256) residual_kernel(const ElemDev<real>* __restrict__ elems,
                                                        int nchunk) {
   const ElemDev<real>& e = elems[blockIdx.z];
@@ -572,7 +576,7 @@ __global__ void __launch_bounds__(256) residual_kernel(const ElemDev<real>* __re
       for (int i = (beg >> 2) + threadIdx.x; i < (end >> 2); i += blockDim.x) {
         const float4 x = X4[i], hx = H4[i], v = V4[i];
         const float4 r = make_float4(hx.x - th * x.x, hx.y - th * x.y, hx.z - th * x.z, hx.w - th * x.w);
-        R4[i] = r;
+        if (PART != 1) R4[i] = r;
         s[0] += r.x * r.x + r.y * r.y + r.z * r.z + r.w * r.w;
         s[1] += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
         s[2] += x.x * hx.x + x.y * hx.y + x.z * hx.z + x.w * hx.w;
@@ -582,7 +586,7 @@ __global__ void __launch_bounds__(256) residual_kernel(const ElemDev<real>* __re
       for (int i = beg + threadIdx.x; i < end; i += blockDim.x) {
         const real x = X[i], hx = HX[i];
         const real r = hx - th * x;
-        R[i] = r;
+        if (PART != 1) R[i] = r;
         s[0] += r * r;
         s[1] += x * x;
         s[2] += x * hx;
@@ -592,21 +596,23 @@ __global__ void __launch_bounds__(256) residual_kernel(const ElemDev<real>* __re
     __shared__ float redf[4][8];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
+      if (PART != 0 && (q == 0) != (PART == 2)) continue;
       float v = s[q];
       for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
       if (lane == 0) redf[q][warp] = v;
     }
     __syncthreads();
-    if (threadIdx.x < 4) {
+    if (threadIdx.x < 4 && (PART == 0 || (threadIdx.x == 0) == (PART == 2))) {
       float v = 0.f;
       for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += redf[threadIdx.x][w];
       e.rpart[((size_t)j * nchunk + blockIdx.x) * 4 + threadIdx.x] = (double)v;
     }
   } else {
+#pragma unroll 4
     for (int i = beg + threadIdx.x; i < end; i += blockDim.x) {
       const real x = X[i], hx = HX[i];
       const real r = hx - th * x;
-      R[i] = r;
+      if (PART != 1) R[i] = r;
       s[0] += r * r;
       s[1] += x * x;
       s[2] += x * hx;
@@ -615,11 +621,12 @@ __global__ void __launch_bounds__(256) residual_kernel(const ElemDev<real>* __re
     __shared__ double red[4][8];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
+      if (PART != 0 && (q == 0) != (PART == 2)) continue;
       double v = warp_sum((double)s[q]);
       if (lane == 0) red[q][warp] = v;
     }
     __syncthreads();
-    if (threadIdx.x < 4) {
+    if (threadIdx.x < 4 && (PART == 0 || (threadIdx.x == 0) == (PART == 2))) {
       double v = 0.0;
       for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[threadIdx.x][w];
       e.rpart[((size_t)j * nchunk + blockIdx.x) * 4 + threadIdx.x] = v;
@@ -761,17 +768,13 @@ __global__ void __launch_bounds__(256) shift_kernel(const ElemDev<real>* __restr
   }
 }
 
-// theta_j = 0 (mode 0) or the Rayleigh quotient x.Hx / x.x from the residual
-// partial sums (mode 1), for every column of every active element.
+// theta_j = the Rayleigh quotient x.Hx / x.x from the residual partial sums, for
+// every column of every active element.
 template <class real>
-__global__ void theta_kernel(const ElemDev<real>* __restrict__ elems, int nchunk, int mode) {
+__global__ void theta_kernel(const ElemDev<real>* __restrict__ elems, int nchunk) {
   const ElemDev<real>& e = elems[blockIdx.z];
   if (!e.state[ST_ACTIVE]) return;
   for (int j = threadIdx.x; j < e.m; j += blockDim.x) {
-    if (mode == 0) {
-      e.theta[j] = 0.0;
-      continue;
-    }
     double xx = 0.0, xhx = 0.0;
     for (int c = 0; c < nchunk; ++c) {
       xx += e.rpart[((size_t)j * nchunk + c) * 4 + 1];
@@ -896,8 +899,11 @@ void launch_tsmm(const Batch<real>& b, const TsmmJob<real>& job, cudaStream_t st
 }
 
 template <class real>
-void launch_residual(const Batch<real>& b, int nchunk, cudaStream_t st) {
-  residual_kernel<real><<<dim3(nchunk, b.s.max_m, b.s.nel), 256, 0, st>>>(b.d_elems, nchunk);
+void launch_residual(const Batch<real>& b, int nchunk, cudaStream_t st, int part) {
+  const dim3 grid(nchunk, b.s.max_m, b.s.nel);
+  if (part == 1) residual_kernel<real, 1><<<grid, 256, 0, st>>>(b.d_elems, nchunk);
+  else if (part == 2) residual_kernel<real, 2><<<grid, 256, 0, st>>>(b.d_elems, nchunk);
+  else residual_kernel<real, 0><<<grid, 256, 0, st>>>(b.d_elems, nchunk);
 }
 
 template <class real>
@@ -919,8 +925,8 @@ void launch_shift(const Batch<real>& b, cudaStream_t st) {
 }
 
 template <class real>
-void launch_theta(const Batch<real>& b, int nchunk, int mode, cudaStream_t st) {
-  theta_kernel<real><<<dim3(1, 1, b.s.nel), 128, 0, st>>>(b.d_elems, nchunk, mode);
+void launch_theta(const Batch<real>& b, int nchunk, cudaStream_t st) {
+  theta_kernel<real><<<dim3(1, 1, b.s.nel), 128, 0, st>>>(b.d_elems, nchunk);
 }
 
 template <class real>
@@ -942,11 +948,11 @@ void init_blas_kernels() {
   template void launch_gram<real>(const Batch<real>&, const GramJob<real>&, double*, size_t,         \
                                   cudaStream_t);                                                     \
   template void launch_tsmm<real>(const Batch<real>&, const TsmmJob<real>&, cudaStream_t);           \
-  template void launch_residual<real>(const Batch<real>&, int, cudaStream_t);                        \
+  template void launch_residual<real>(const Batch<real>&, int, cudaStream_t, int);                   \
   template void launch_post_residual<real>(const Batch<real>&, int, int, cudaStream_t);              \
   template void launch_iter_finish<real>(const Batch<real>&, int, cudaStream_t);                    \
   template void launch_restart<real>(const Batch<real>&, cudaStream_t);                              \
-  template void launch_theta<real>(const Batch<real>&, int, int, cudaStream_t);                     \
+  template void launch_theta<real>(const Batch<real>&, int, cudaStream_t);                          \
   template void launch_shift<real>(const Batch<real>&, cudaStream_t);
 DGDFT_INST(double)
 DGDFT_INST(float)

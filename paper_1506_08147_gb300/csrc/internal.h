@@ -144,9 +144,10 @@ void init_blas_kernels();
 // false where the job has more columns than the kernel takes
 bool launch_update_dig(const Batch<double>& b, const TsmmJob<double>& job, cudaStream_t st);
 
-// Residual R = HX - X diag(theta) into W, with per-column partial sums.
+// Residual R = HX - X diag(theta) into W, with per-column partial sums; part 1:
+// only the sums that need no theta, part 2: only R and its norm.
 template <class real>
-void launch_residual(const Batch<real>& b, int nchunk, cudaStream_t st);
+void launch_residual(const Batch<real>& b, int nchunk, cudaStream_t st, int part = 0);
 // Reduces the partial sums: residual norms, kinetic energies for Teter,
 // convergence and iteration bookkeeping.
 template <class real>
@@ -164,9 +165,9 @@ void launch_iter_finish(const Batch<real>& b, int set_p, cudaStream_t st);
 // iteration (post_residual decides d).
 template <class real>
 void launch_shift(const Batch<real>& b, cudaStream_t st);
-// theta = 0 (mode 0) or the Rayleigh quotients from the residual sums (mode 1)
+// theta = the Rayleigh quotients from the residual sums
 template <class real>
-void launch_theta(const Batch<real>& b, int nchunk, int mode, cudaStream_t st);
+void launch_theta(const Batch<real>& b, int nchunk, cudaStream_t st);
 
 // dense.cu: FP64 Rayleigh-Ritz on one CTA per task.
 enum { RR_FIXED = 0, RR_INITIAL = 1, RR_LOBPCG = 2 };

@@ -1128,11 +1128,10 @@ template <class real> struct Wave {
     // the FP32 stage's block, projected by the FP64 stage's mask
     if (cutoff()) project_block(BX, st);
     launch_apply_h<real>(batch, bref<real>(BX), bref<real>(BHX), 0, st, fwd64());
-    launch_theta<real>(batch, rnchunk, 0, st);
-    launch_residual<real>(batch, rnchunk, st);
-    launch_theta<real>(batch, rnchunk, 1, st);
+    launch_residual<real>(batch, rnchunk, st, 1);
+    launch_theta<real>(batch, rnchunk, st);
     if (batch.s.max_nproj > 0) launch_proj_coef<real>(batch, bref<real>(BX), 0, st);
-    launch_residual<real>(batch, rnchunk, st);
+    launch_residual<real>(batch, rnchunk, st, 2);
     if (cutoff()) project_residual(st);
     launch_post_residual<real>(batch, rnchunk, 1 << 30, st);
     CK(cudaGetLastError());
