@@ -9,7 +9,7 @@
 // ms; with pairs on the FP32 pipes (the mixed form) a fifth of that.  Here the
 // integer instructions of the digit splitting and of reading the sums do, and
 // the products issued beside them.  Four elements, an SCF step: the Gram
-// products 77 -> 8 ms (nine launches), the updates 45 -> 10 (14); one element of
+// products 77 -> 8 ms (nine launches), the updates 45 -> 10 (14 launches); one element of
 // 4,096 rows and 16 columns: 31 -> 12.5 us and 36 -> 13 us a launch, so the
 // SIMT kernels are not kept for small blocks either.  The orthonormalisation
 // (36 elements of 13,440 points, 40 columns): Gram 0.97 and update 1.30 ms a
@@ -215,12 +215,16 @@ __global__ void __launch_bounds__(DIG_THREADS, 1) update_dig_kernel(Src src, int
   dig_open(cta, bar, &slot);
   const long long total = (long long)nel * nct * tiles, per = (total + gridDim.x - 1) / gridDim.x;
   const long long end = min(total, (blockIdx.x + 1) * per);
-  long long have = -1;
+  long long have = -1, known = -1;
   int K = 0;
+  UpdDesc d;  // of the element and output columns at hand
   for (long long it = blockIdx.x * per; it < end; ++it) {
     const int el = (int)(it / ((long long)nct * tiles)), rem = (int)(it - (long long)el * nct * tiles);
     const int ct = rem / tiles, tile = rem - ct * tiles;
-    const UpdDesc d = src(el, ct * NB);
+    if (it / tiles != known) {
+      known = it / tiles;
+      d = src(el, ct * NB);
+    }
     const int r0 = tile * DIG_M, rows = d.rows;
     if (d.nout <= 0 || r0 >= rows) continue;
     const int nB = min(NB, d.nout), ldy = d.ldy;
