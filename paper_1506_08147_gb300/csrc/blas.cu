@@ -664,7 +664,7 @@ __global__ void __launch_bounds__(256) rnorm_kernel(const ElemDev<real>* __restr
 // Residual norms, kinetic energies, convergence.  One CTA per element; a thread
 // takes one of a column's four sums, or an eighth of its projector sum (with a
 // thread per column the chain of FP64 operations took 64 us at m = 48,
-// MEASURED_PR).
+// this one 22 us).
 constexpr int PR_COLS = 64, PR_PARTS = 8;
 
 template <class real>
